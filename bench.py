@@ -875,7 +875,7 @@ def _ws_conv_roofline(B, n, stream):
     achieved = flops / ms / 1e9
     return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": None, "peak_source": src,
-            "kernel": f"conv3x3_fwd_tc<32, wide> {cin}->{cout} on {B} x {n}^2 (tcgen05.mma kind::f16, BF16 operands, "
+            "kernel": f"conv3x3_fwd<32, 32> {cin}->{cout} on {B} x {n}^2 (tcgen05.mma kind::f16, BF16 operands, "
                       "FP32 accumulator in TMEM)"}
 
 

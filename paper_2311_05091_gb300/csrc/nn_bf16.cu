@@ -11,11 +11,14 @@
 // both operands MN-major; activations are rounded to BF16 as they enter a convolution,
 // weights are kept as a BF16 copy of FP32 master weights.  Weight layout: wt[tap][cout][cin], tap = 3 ky + kx, so a
 // pair of input channels is one 32-bit word.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "../../include/lbm_nn.h"
 
@@ -32,25 +35,35 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // ---------------------------------------------------------------------------
 // forward: y[p][co] = act(b[co] + sum_{tap, ci} x[p + shift(tap)][ci] wt[tap][co][ci])
 //
-// Implicit GEMM on the 5th-generation tensor cores: D (128 output pixels x N
-// output channels, FP32 in TMEM) += A_tap (128 x 16 input channels, BF16) *
-// B_tap^T (N x 16) for the nine taps and every chunk of 16 input channels.
-// The 128 pixels of a CTA are R image rows of W = 128 / R columns (W = 128,
-// 64, 32 or 16, the smallest that covers the image width, so narrow levels
-// keep the M = 128 tile full).  Per chunk the CTA stages in shared memory, as
-// BF16 in the canonical K-major layout without swizzle (core matrices of 8
-// rows x 16 bytes; rows 16 bytes apart, 8-row groups 128 bytes apart, the
-// two 8-channel halves of the chunk LBO bytes apart):
-//   A: for each column offset kx, rows y0 - 1 .. y0 + R of the input at
-//      columns x0 + kx - 1 .. x0 + kx - 2 + W (zero outside the image), so
-//      that tap (ky, kx) is the 128-row window starting at row ky of copy kx;
-//   B: the weights of all nine taps, [tap][half][co].
-// One thread issues the nine tcgen05.mma of the chunk and commits them to the
-// stage's mbarrier; with two stages the next chunk is staged while the tensor
-// cores work; a stage is refilled only after the bounded wait for the
-// products that read it.  The epilogue reads the accumulator with tcgen05.ld
-// (warp w owns TMEM lanes 32 w .. 32 w + 31 = pixels), adds the bias, applies
-// the ReLU and stores FP32.  grid (segments, cout / N), 128 threads.
+// Implicit GEMM on the 5th-generation tensor cores: D (128 positions x N output channels, FP32 in TMEM) +=
+// A_tap (128 x 16 input channels, BF16) * B_tap^T (N x 16) for every chunk of 16 input channels and, inside it, the
+// nine taps (this order fixes the rounding of the sums).
+//
+// Positions, not pixels.  A work item is a block of R image rows x Wt columns, staged with one halo row above and
+// below and one halo column on each side as a flat sequence of positions of pitch Wt + 2, zero outside the image.
+// Output position m = row * pitch + column reads position m + ky * pitch + kx for tap (ky, kx), so one staged copy
+// serves all nine taps of any image width: the A operand of a tap is the window of 128 consecutive positions that
+// starts ky * pitch + kx positions further, in the canonical K-major layout without swizzle (16 bytes per position
+// and 8-channel group; core matrices 128 bytes apart along M, channel groups LBO apart).  The two outputs per row
+// that fall on the halo columns are dropped (3 % of the products at Wt = 64).  The images of the batch are one tall
+// image with a zero row between them, so blocks of rows run across image borders.
+//
+// One persistent CTA per SM, three roles that run concurrently:
+//   producers:  look up each staged position's pixel (a table built once per item), load FP32 activations 32 bytes
+//               per thread, round to BF16 into the stage (16-byte stores, free of bank conflicts); one thread starts
+//               the TMA copy of the stage's weights, [tap][co][KC channels] in the matching 64- or 32-byte swizzle;
+//   products:   one thread issues the tcgen05.mma of a stage and commits them to the barrier that frees it;
+//   epilogue:   reads a finished accumulator (tcgen05.ld), adds the bias, applies the ReLU, transposes through
+//               shared memory and stores whole 128-byte lines.
+// Stages of KC channels form a ring over items; the accumulators have two sets, so an item's products overlap the
+// previous item's epilogue.  Every barrier wait is bounded; a give-up sets g_nn_fault and ends the CTA.
+//
+// What bounds it: the wide levels HBM (403 MB for 64 -> 32 on 16 x 256^2: 60 us at copy speed), the deep ones shared
+// memory (an M = 128, K = 16 product reads 4 KB of A, 32 cycles, whatever N) and the pipeline's latency per stage.
+// Measured (GB300, 16 images; the kernel before staged every tile between two CTA barriers, without overlap):
+// 64 -> 32 on 256^2 331 -> 109 us, 128 -> 128 on 64^2 137 -> 31 us, 256 -> 256 on 32^2 101 -> 31 us, one image of the
+// last 54 -> 15 us.  12 producer warps with four 32-byte loads each in flight: 824 us over the network's seventeen
+// forward and data-gradient shapes, against 856 with 8 warps and 830 with 16.
 // ---------------------------------------------------------------------------
 __device__ unsigned int g_nn_fault = 0;    // set when a bounded wait on the tensor cores gave up
 
@@ -62,9 +75,38 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
          (1ull << 46);
 }
 
+// the same for K-major rows of `row` bytes (32 or 64) in TMA's swizzle of that width, rows contiguous: 8-row groups
+// 8 row bytes apart; a later K = 16 slice of the row starts 32 bytes further
+template <int row>
+__device__ __forceinline__ uint64_t umma_desc_sw(uint32_t addr) {
+  static_assert(row == 32 || row == 64, "swizzle widths used here");
+  return (uint64_t)((addr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)((8 * row) >> 4) << 32) | (1ull << 46) |
+         ((row == 64 ? 4ull : 6ull) << 61);
+}
+
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both K-major, M x N
 __host__ __device__ constexpr uint32_t umma_idesc(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+}
+
+// D (TMEM) = or += A B^T, one K = 16 product of kind::f16
+__device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
+// the products issued so far arrive on an mbarrier when they are done
+__device__ __forceinline__ void umma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar));
+}
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 // bounded wait for the completion of phase `parity` of an mbarrier; false when it gave up
@@ -74,57 +116,80 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(bar), "r"(parity));
+        : "r"(bar), "r"(parity)
+        : "memory");
   return done != 0;
 }
 
-constexpr int kTcM = 128;
-constexpr int kTcThreads = 256;   // 8 warps stage the tiles; warps w and w + 4 share TMEM lane quarter w % 4
-constexpr int kFwdBatch = 3;      // staging items whose loads a thread has in flight at once
+constexpr int kCvEpi = 8;                          // epilogue warps, two per TMEM lane quarter
+constexpr int kCvMma = kCvEpi;                     // the warp that issues the products
+constexpr int kCvProd = 12;                        // producer warps
+constexpr int kCvThreads = 32 * (kCvEpi + 1 + kCvProd);
+constexpr int kCvBatch = 4;                        // 8-channel groups (32 bytes) a producer thread has in flight
+constexpr int kCvMaxStages = 6;
+constexpr int kCvSmem = 227 * 1024;                // shared memory a CTA may use
+constexpr int kCvHead = 512 + kCvEpi * 4096;       // barriers, epilogue transposition buffers
 
-// (A, B) tiles in S stages: with two, one chunk is staged while the tensor cores multiply the previous one.
-// Two stages pay only where the tiles are small enough to keep several CTAs per SM (measured on GB300: wide
-// images with N <= 64 gain 5-12 %, the 128-channel tiles lose up to 35 % when their occupancy halves).
-// A holds at most 24 KB: WIDE 2 x 3 x 130 x 16 bytes; otherwise 6 (R + 2) W 16 <= 24576 bytes (R = 2).
-template <int N, bool WIDE>
-struct FwdTcSmem {
-  static constexpr int S = (WIDE && N <= 64) ? 2 : 1;
-  static constexpr int kA = WIDE ? 13312 : 24576;
-  static constexpr int kB = 9 * 2 * N * 16;
-  static constexpr int kStage = kA + kB;
-  static constexpr int bytes() { return S * kStage + 64; }
+// How a convolution is cut into work items (host).
+struct FwdPlan {
+  int N, KC;                 // output channels per item, input channels per stage
+  int Wt, pitch, strips;     // columns per item, staged columns, column strips
+  int R, T;                  // rows per item, 128-position tiles per item
+  int Pn;                    // staged positions allocated per channel group (Pn % 8 == 2: conflict-free stores)
+  int stages, stage_bytes, smem, tmem;
+  int blocks, items;         // row blocks of the tall image; items = blocks * strips * (cout / N)
 };
 
-// WIDE (one image row of 128 columns per CTA): a single copy of the three input rows with one halo column each
-// side, [half][row][column] x 16 bytes; the window of tap (ky, kx) starts at row ky, column kx, i.e. 16 kx bytes
-// further, and its 128 rows stay 16 bytes apart.  Otherwise (R > 1 rows per CTA) the rows of the window cross
-// image rows, so the input is staged once per column offset kx as described above.
-template <int N, bool WIDE>
-__global__ void __launch_bounds__(kTcThreads) conv3x3_fwd_tc(const float* __restrict__ x,
-                                                           const __nv_bfloat16* __restrict__ wt,
-                                                           const float* __restrict__ bias, float* __restrict__ y,
-                                                           int n, int h, int w, int cin, int cout, int relu,
-                                                           int R) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  using SM = FwdTcSmem<N, WIDE>;
-  constexpr int S = SM::S;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + S * SM::kStage);   // one mbarrier per stage
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int W = kTcM / R;
-  const int segx = (w + W - 1) / W, segy = (h + R - 1) / R;
-  const int sx = blockIdx.x % segx, sy = (blockIdx.x / segx) % segy, img = blockIdx.x / (segx * segy);
-  const int x0 = sx * W, y0 = sy * R;
-  const int co0 = blockIdx.y * N;
-  const uint32_t bar0 = smem_addr(bar);
+struct FwdArgs {
+  const float* x;
+  const float* bias;
+  float* y;
+  int n, h, w, cin, cout, relu;
+  FwdPlan p;
+};
 
-  if (warp == 0) {
+// barrier of the producer warps with the conjunction of their predicates
+__device__ __forceinline__ bool producers_and(bool ok) {
+  int all;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.and.pred q, 1, %2, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(all)
+      : "r"((int)ok), "n"(32 * kCvProd)
+      : "memory");
+  return all != 0;
+}
+
+template <int N, int KC>
+__global__ void __launch_bounds__(kCvThreads, 1)
+    conv3x3_fwd(const FwdArgs a, const __grid_constant__ CUtensorMap wmap) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  constexpr int KG = KC / 8;                        // channel groups per stage
+  constexpr int kW = 9 * N * KC * 2;                // bytes of a stage's weights
+  const FwdPlan& p = a.p;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int S = p.stages;
+  // barriers: activations staged[S], weights landed[S], stage free[S], accumulator ready[2], accumulator free[2]
+  const uint32_t b_full = smem_addr(smem), b_w = b_full + 8 * kCvMaxStages, b_empty = b_w + 8 * kCvMaxStages,
+                 b_acc = b_empty + 8 * kCvMaxStages, b_free = b_acc + 16;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + 24 * kCvMaxStages + 32);
+  float* tbuf = reinterpret_cast<float*>(smem + 512);
+  unsigned char* stage0 = smem + kCvHead;
+
+  if (warp == kCvMma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
-                 "r"(N < 32 ? 32 : N));
+                 "r"(p.tmem));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int k = 0; k < S; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8 * k), "r"(1));
+    for (int k = 0; k < S; ++k) {
+      mbar_init(b_full + 8 * k, 32 * kCvProd);
+      mbar_init(b_w + 8 * k, 1);
+      mbar_init(b_empty + 8 * k, 1);
+    }
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(b_acc + 8 * k, 1);
+      mbar_init(b_free + 8 * k, 32 * kCvEpi);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
@@ -132,122 +197,257 @@ __global__ void __launch_bounds__(kTcThreads) conv3x3_fwd_tc(const float* __rest
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tslot);
 
-  const int rows = R + 2;
-  const int pitch = WIDE ? W + 2 : W;                    // staged columns per row
-  const uint32_t lbo_a = (uint32_t)(rows * pitch * 16), lbo_b = (uint32_t)(N * 16);
-  const int nchunks = cin / 16;
+  const int ntile = a.cout / N;
+  const int nst = a.cin / KC;
+  const int rows_all = a.n * (a.h + 1) - 1;         // rows of the tall image
   bool ok = true;
-  for (int c = 0; c < nchunks; ++c) {
-    const int ci0 = c * 16, st = c % S;
-    unsigned char* sA = smem + st * SM::kStage;
-    unsigned char* sB = sA + SM::kA;
-    // the products of chunk c - S read this stage: wait for them (phase (c - S) / S of this stage's barrier)
-    if (c >= S) ok = ok && mbar_wait(bar0 + 8 * st, ((c - S) / S) & 1);
-    // B: the BF16 weights of the nine taps, copied asynchronously (16 bytes, no register round trip)
-    for (int e = tid; e < 18 * N; e += kTcThreads) {
-      const int co = e % N, kc = (e / N) & 1, tap = e / (2 * N);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(sB + ((tap * 2 + kc) * N + co) * 16)),
-                   "l"(wt + ((long long)tap * cout + co0 + co) * cin + ci0 + 8 * kc)
-                   : "memory");
-    }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-    // A: WIDE, one copy of rows y0 - 1 .. y0 + 1 at columns x0 - 1 .. x0 + 128; else one copy per kx.  The global
-    // loads of kFwdBatch items per thread are issued before their conversions and shared stores (a store may not
-    // be moved above a later load through pointers that could alias)
-    const int nA = (WIDE ? 2 : 6) * rows * pitch;
-    for (int e0 = 0; e0 < nA; e0 += kFwdBatch * kTcThreads) {
-      float4 pv[kFwdBatch], qv[kFwdBatch];
-      int off[kFwdBatch];   // destination byte offset from sA, -1: none
+
+  if (warp > kCvMma) {
+    // ---- producers ----
+    const int tp = tid - 32 * (kCvMma + 1);
+    constexpr int TP = 32 * kCvProd;
+    constexpr int PP = TP / KG;                     // positions per pass of the producer threads
+    const int kg = tp % KG, q0 = tp / KG;
+    int* tab = reinterpret_cast<int*>(stage0 + S * p.stage_bytes);   // staged position -> pixel, -1: zero
+    int it = 0;                                     // stage count over all items
+    for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
+      // the previous item's table is no longer read; producers leave together when one gave up
+      if (!(ok = producers_and(ok))) break;
+      const int ct = item % ntile, rest = item / ntile;
+      const int x0 = rest % p.strips * p.Wt, row0 = rest / p.strips * p.R;
+      const int NP = (min(p.R, rows_all - row0) + 2) * p.pitch;
+      // the positions' pixels once per item (the same for every channel chunk), shared by the KG threads of a position
+      for (int q = tp; q < NP; q += TP) {
+        const int r = q / p.pitch, xx = x0 - 1 + q - r * p.pitch;
+        const unsigned row = (unsigned)(row0 + r + a.h);      // tall-image row of the halo above, one image further
+        const int img = (int)(row / (unsigned)(a.h + 1)), yy = (int)(row - (unsigned)img * (a.h + 1));
+        tab[q] = (yy < a.h && (unsigned)xx < (unsigned)a.w) ? ((img - 1) * a.h + yy) * a.w + xx : -1;
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(TP) : "memory");
+      for (int s = 0; s < nst; ++s, ++it) {
+        const int st = it % S;
+        unsigned char* sw = stage0 + st * p.stage_bytes;
+        if (it >= S && !mbar_wait(b_empty + 8 * st, (uint32_t)((it / S - 1) & 1))) {
+          ok = false;
+          break;
+        }
+        if (tp == 0) {                              // the weights of the nine taps: one TMA tile
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(b_w + 8 * st), "r"(kW)
+                       : "memory");
+          asm volatile(
+              "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+              "%4}], [%5];\n" ::"r"(smem_addr(sw)),
+              "l"(reinterpret_cast<unsigned long long>(&wmap)), "r"(s * KC), "r"(ct * N), "r"(0), "r"(b_w + 8 * st)
+              : "memory");
+        }
+        const float* src = a.x + s * KC + 8 * kg;
+        unsigned char* dst = sw + kW + kg * p.Pn * 16;
+        for (int q = q0; q < NP; q += PP * kCvBatch) {
+          float4 v[kCvBatch][2];
 #pragma unroll
-      for (int k = 0; k < kFwdBatch; ++k) {
-        const int e = e0 + k * kTcThreads + tid;
-        off[k] = -1;
-        pv[k] = qv[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (e < nA) {
-          const int px = e % pitch, r = (e / pitch) % rows, kc = (e / (pitch * rows)) & 1;
-          const int kx = WIDE ? 0 : e / (pitch * rows * 2);
-          const int yy = y0 + r - 1, xc = x0 + px + kx - 1;
-          off[k] = (((kx * 2 + kc) * rows + r) * pitch + px) * 16;
-          if (yy >= 0 && yy < h && xc >= 0 && xc < w) {
-            const float* src = x + (((long long)img * h + yy) * w + xc) * cin + ci0 + 8 * kc;
-            pv[k] = __ldg(reinterpret_cast<const float4*>(src));
-            qv[k] = __ldg(reinterpret_cast<const float4*>(src + 4));
+          for (int u = 0; u < kCvBatch; ++u) {
+            const int qq = q + u * PP;
+            const int pix = qq < NP ? tab[qq] : -1;
+            v[u][0] = v[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (pix >= 0) {
+              const float4* at = reinterpret_cast<const float4*>(src + (long long)pix * a.cin);
+              v[u][0] = __ldg(at);
+              v[u][1] = __ldg(at + 1);
+            }
           }
+#pragma unroll
+          for (int u = 0; u < kCvBatch; ++u)
+            if (q + u * PP < NP)
+              *reinterpret_cast<uint4*>(dst + (q + u * PP) * 16) =
+                  make_uint4(pack_bf16(v[u][0].x, v[u][0].y), pack_bf16(v[u][0].z, v[u][0].w),
+                             pack_bf16(v[u][1].x, v[u][1].y), pack_bf16(v[u][1].z, v[u][1].w));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // stores visible to the tensor cores
+        mbar_arrive(b_full + 8 * st);
+      }
+    }
+    // leave no copy in flight: the last weight tiles issued (landed already unless a wait gave up)
+    if (tp == 0)
+      for (int k = 0; k < S && k < it; ++k) (void)mbar_wait(b_w + 8 * ((it - 1 - k) % S), (uint32_t)(((it - 1 - k) / S) & 1));
+  } else if (warp == kCvMma) {
+    // ---- products: one thread ----
+    if (lane == 0) {
+      constexpr uint32_t idesc = umma_idesc(128, N);
+      const uint32_t lbo = (uint32_t)p.Pn * 16;
+      int it = 0, na = 0;
+      for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++na) {
+        const int acc = na & 1;
+        if (na >= 2 && !mbar_wait(b_free + 8 * acc, (uint32_t)((na / 2 - 1) & 1))) {
+          ok = false;
+          break;
+        }
+        const int rows = min(p.R, rows_all - item / (ntile * p.strips) * p.R);
+        const int T = ((rows - 1) * p.pitch + p.Wt + 127) / 128;
+        const uint32_t d0 = tmem + (uint32_t)(acc * p.T * N);
+        for (int s = 0; s < nst; ++s, ++it) {
+          const int st = it % S;
+          if (!mbar_wait(b_w + 8 * st, (uint32_t)((it / S) & 1)) || !mbar_wait(b_full + 8 * st, (uint32_t)((it / S) & 1))) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t sw = smem_addr(stage0 + st * p.stage_bytes), sx = sw + kW;
+          for (int t = 0; t < T; ++t) {
+#pragma unroll
+            for (int sub = 0; sub < KC / 16; ++sub) {
+              const uint32_t ax = sx + (uint32_t)(2 * sub * p.Pn + t * 128) * 16;
+#pragma unroll
+              for (int tap = 0; tap < 9; ++tap)
+                umma_f16(d0 + t * N, umma_desc(ax + (uint32_t)((tap / 3) * p.pitch + tap % 3) * 16, lbo, 128),
+                         umma_desc_sw<2 * KC>(sw + tap * N * KC * 2 + 32 * sub), idesc, (s > 0 || sub > 0 || tap > 0) ? 1u : 0u);
+            }
+          }
+          umma_commit(b_empty + 8 * st);
+        }
+        if (ok) umma_commit(b_acc + 8 * acc);
+      }
+      // leave no product in flight: the last commits of the stages
+      for (int k = 0; k < S && k < it; ++k) {
+        const int last = it - 1 - k;
+        (void)mbar_wait(b_empty + 8 * (last % S), (uint32_t)((last / S) & 1));
+      }
+    }
+    __syncwarp();
+  } else {
+    // ---- epilogue ----
+    const int quarter = warp & 3;
+    float* buf = tbuf + warp * 1024;                // 32 pixels x 32 channels, 16-byte chunks swizzled by pixel
+    const int j = lane & 7;                         // lane j + 8 k stores channels 4 j .. of pixels k, k + 4, ...
+    int na = 0;
+    for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++na) {
+      const int acc = na & 1;
+      const int ct = item % ntile, rest = item / ntile;
+      const int x0 = rest % p.strips * p.Wt, row0 = rest / p.strips * p.R;
+      const int rows = min(p.R, rows_all - row0);
+      const int T = ((rows - 1) * p.pitch + p.Wt + 127) / 128;
+      if (!mbar_wait(b_acc + 8 * acc, (uint32_t)((na / 2) & 1))) {
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      // (tile, 32 channels) units alternate between the two warps of a lane quarter
+      for (int unit = warp >> 2; unit < T * (N / 32); unit += 2) {
+        const int t = unit / (N / 32), c0 = unit % (N / 32) * 32;
+        // output pixel of this lane's TMEM row, -1: a halo column or row
+        const int m = t * 128 + quarter * 32 + lane;
+        const int r = m / p.pitch, c = m - r * p.pitch;
+        const unsigned row = (unsigned)(row0 + r);
+        const int img = (int)(row / (unsigned)(a.h + 1)), yy = (int)(row - (unsigned)img * (a.h + 1));
+        const int pix = (r < rows && yy < a.h && c < p.Wt && x0 + c < a.w) ? (img * a.h + yy) * a.w + x0 + c : -1;
+        const int ch = ct * N + c0 + 4 * j;
+        float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (a.bias) bv = make_float4(a.bias[ch], a.bias[ch + 1], a.bias[ch + 2], a.bias[ch + 3]);
+        {
+          uint32_t v[32];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+              "%15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+                "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+                "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+              : "r"(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((acc * p.T + t) * N + c0)));
+          asm volatile("tcgen05.wait::ld.sync.aligned;");
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            *reinterpret_cast<uint4*>(buf + lane * 32 + ((j ^ (lane & 7)) * 4)) =
+                make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int px = 4 * i + (lane >> 3);
+            const int at = __shfl_sync(0xffffffffu, pix, px);   // whole 128-byte lines
+            float4 o = *reinterpret_cast<const float4*>(buf + px * 32 + ((j ^ (px & 7)) * 4));
+            o = make_float4(o.x + bv.x, o.y + bv.y, o.z + bv.z, o.w + bv.w);
+            if (a.relu) o = make_float4(fmaxf(o.x, 0.f), fmaxf(o.y, 0.f), fmaxf(o.z, 0.f), fmaxf(o.w, 0.f));
+            if (at >= 0) *reinterpret_cast<float4*>(a.y + (long long)at * a.cout + ch) = o;
+          }
+          __syncwarp();
         }
       }
-#pragma unroll
-      for (int k = 0; k < kFwdBatch; ++k)
-        if (off[k] >= 0)
-          *reinterpret_cast<uint4*>(sA + off[k]) =
-              make_uint4(pack_bf16(pv[k].x, pv[k].y), pack_bf16(pv[k].z, pv[k].w), pack_bf16(qv[k].x, qv[k].y),
-                         pack_bf16(qv[k].z, qv[k].w));
-    }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;");       // generic-proxy stores visible to the tensor cores
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (tid == 0 && ok) {
-      constexpr uint32_t idesc = umma_idesc(kTcM, N);
-#pragma unroll 1
-      for (int tap = 0; tap < 9; ++tap) {
-        const int ky = tap / 3, kx = tap % 3;
-        const uint64_t ad = WIDE ? umma_desc(smem_addr(sA + (ky * pitch + kx) * 16), lbo_a, 128)
-                                 : umma_desc(smem_addr(sA + ((kx * 2) * rows + ky) * W * 16), lbo_a, 128);
-        const uint64_t bd = umma_desc(smem_addr(sB + tap * 2 * N * 16), lbo_b, 128);
-        const uint32_t acc = (c > 0 || tap > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 8 * st));
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      mbar_arrive(b_free + 8 * acc);
     }
   }
-  // the last commit completes after every product issued before it
-  ok = ok && mbar_wait(bar0 + 8 * ((nchunks - 1) % S), ((nchunks - 1) / S) & 1);
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (ok) {
-    const int q = warp & 3;                                // TMEM lane quarter of this warp
-    const int m = q * 32 + lane;
-    const int yo = y0 + m / W, xo = x0 + m % W;
-    const bool valid = yo < h && xo < w;
-    float* dst = y + (((long long)img * h + yo) * w + xo) * cout + co0;
-    constexpr int HALF = N / 2;                            // warps 0-3 take columns 0 .. N/2, warps 4-7 the rest
-#pragma unroll 1
-    for (int c0 = (warp >> 2) * HALF; c0 < (warp >> 2) * HALF + HALF; c0 += 16) {
-      uint32_t r[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-          "%14, %15}, [%16];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0));
-      asm volatile("tcgen05.wait::ld.sync.aligned;");
-      if (valid) {
-#pragma unroll
-        for (int j = 0; j < 16; j += 4) {
-          float4 o;
-          o.x = __uint_as_float(r[j]) + (bias ? bias[co0 + c0 + j] : 0.f);
-          o.y = __uint_as_float(r[j + 1]) + (bias ? bias[co0 + c0 + j + 1] : 0.f);
-          o.z = __uint_as_float(r[j + 2]) + (bias ? bias[co0 + c0 + j + 2] : 0.f);
-          o.w = __uint_as_float(r[j + 3]) + (bias ? bias[co0 + c0 + j + 3] : 0.f);
-          if (relu) {
-            o.x = fmaxf(o.x, 0.f);
-            o.y = fmaxf(o.y, 0.f);
-            o.z = fmaxf(o.z, 0.f);
-            o.w = fmaxf(o.w, 0.f);
-          }
-          *reinterpret_cast<float4*>(dst + c0 + j) = o;
-        }
-      }
-    }
-  } else if (tid == 0) {
-    atomicExch(&g_nn_fault, 1u);
-  }
+  if (!ok) atomicExch(&g_nn_fault, 1u);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(N < 32 ? 32 : N));
+  if (warp == kCvMma) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem));
+}
+
+// Tensor map of the weights: boxes of KC input channels x N output channels x nine taps.
+bool weight_map(CUtensorMap* map, const void* wt, int cin, int cout, int N, int KC) {
+  static std::atomic<void*> entry{nullptr};
+  void* fn = entry.load(std::memory_order_acquire);
+  if (!fn) {
+    cudaDriverEntryPointQueryResult qr;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &qr) != cudaSuccess ||
+        qr != cudaDriverEntryPointSuccess || !fn)
+      return false;
+    entry.store(fn, std::memory_order_release);
+  }
+  const cuuint64_t dims[3] = {(cuuint64_t)cin, (cuuint64_t)cout, 9};
+  const cuuint64_t strides[2] = {(cuuint64_t)cin * 2, (cuuint64_t)cin * cout * 2};
+  const cuuint32_t box[3] = {(cuuint32_t)KC, (cuuint32_t)N, 9};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn)(
+             map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(wt), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, KC == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Cuts the convolution into items: among the channel tiles N, the numbers of column strips (of at most 128 columns)
+// and the tiles per item, the least modelled time: waves of one CTA per SM x the largest of the product time (32
+// cycles per M = 128 product up to N = 64, then N / 2), the staging time and the store time (32 bytes per SM and
+// cycle each), plus a fixed latency per item and stage.  Small images get many small items, so that one image of a
+// deep level still reaches half of the SMs; large ones get items of up to 1024 positions, whose halo costs least.
+FwdPlan fwd_plan(int n, int h, int w, int cin, int cout, int sms) {
+  FwdPlan best{};
+  double best_cost = -1.0;
+  const int KC = cin % 32 == 0 ? 32 : 16;
+  const int rows_all = n * (h + 1) - 1;
+  for (int N = 32; N <= 128; N *= 2) {
+    if (cout % N) continue;
+    const int k0 = (w + 127) / 128;
+    for (int k = k0; k <= k0 + 3 && k <= w; ++k) {
+      const int Wt = (w + k - 1) / k, pitch = Wt + 2, strips = (w + Wt - 1) / Wt;
+      for (int T = 1; T * N <= 256; ++T) {
+        if (128 * T < Wt) continue;
+        FwdPlan p{};
+        p.N = N;
+        p.KC = KC;
+        p.Wt = Wt;
+        p.pitch = pitch;
+        p.strips = strips;
+        p.T = T;
+        p.R = std::min((128 * T - Wt) / pitch + 1, rows_all);
+        p.blocks = (rows_all + p.R - 1) / p.R;
+        p.R = (rows_all + p.blocks - 1) / p.blocks;
+        p.Pn = 128 * T + 2 * pitch + 2;
+        p.Pn += (10 - p.Pn % 8) % 8;                              // Pn % 8 == 2
+        p.stage_bytes = (KC / 8) * p.Pn * 16 + 18 * N * KC;
+        p.stage_bytes = (p.stage_bytes + 511) / 512 * 512;        // the weights' swizzle pattern repeats every 512 bytes
+        p.stages = std::min(kCvMaxStages, (kCvSmem - kCvHead - 4 * p.Pn) / p.stage_bytes);
+        if (p.stages < 2) continue;
+        p.smem = kCvHead + p.stages * p.stage_bytes + 4 * p.Pn;
+        p.tmem = 32;
+        while (p.tmem < 2 * T * N) p.tmem *= 2;
+        p.items = p.blocks * strips * (cout / N);
+        const double mma = (double)T * 9 * (cin / 16) * std::max(32, N / 2);
+        const double load = ((double)(p.R + 2) * pitch * cin * 4 + 18.0 * cin * N) / 32.0;
+        const double out = (double)T * N * 128 * 4 / 32.0;
+        const double item = std::max(std::max(mma, load), out) + 300.0;
+        const double cost = (double)((p.items + sms - 1) / sms) * item + 400.0 * (cin / KC);
+        if (best_cost < 0 || cost < best_cost) best = p, best_cost = cost;
+      }
+    }
+  }
+  return best;
 }
 
 // ---------------------------------------------------------------------------
@@ -887,45 +1087,45 @@ int lbm_nn_conv3x3(const float* x, const void* wt_bf16, const float* bias, float
                    int cout, int relu, void* stream) {
   if (!x || !wt_bf16 || !y || n < 1 || h < 1 || w < 1 || cin < 16 || cin % 16 || cout < 32 || cout % 32) return -1;
   // the opt-in above 48 KB of shared memory is a per-device attribute: set it once for each device used
-  static unsigned long long attr_set = 0;
+  static std::atomic<unsigned long long> attr_set{0};
+  static std::atomic<int> sm_count[64];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -3;
-  if (!(attr_set & (1ull << dev))) {
-    bool good = true;
-    auto opt_in = [&](const void* fn, int bytes) {
-      good = good && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
-    };
-    opt_in((const void*)conv3x3_fwd_tc<128, true>, FwdTcSmem<128, true>::bytes());
-    opt_in((const void*)conv3x3_fwd_tc<64, true>, FwdTcSmem<64, true>::bytes());
-    opt_in((const void*)conv3x3_fwd_tc<32, true>, FwdTcSmem<32, true>::bytes());
-    opt_in((const void*)conv3x3_fwd_tc<128, false>, FwdTcSmem<128, false>::bytes());
-    opt_in((const void*)conv3x3_fwd_tc<64, false>, FwdTcSmem<64, false>::bytes());
-    opt_in((const void*)conv3x3_fwd_tc<32, false>, FwdTcSmem<32, false>::bytes());
-    if (!good) return -3;
-    attr_set |= 1ull << dev;
+  if (!(attr_set.load(std::memory_order_acquire) & (1ull << dev))) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return -3;
+    for (const void* fn : {(const void*)conv3x3_fwd<32, 16>, (const void*)conv3x3_fwd<32, 32>,
+                           (const void*)conv3x3_fwd<64, 16>, (const void*)conv3x3_fwd<64, 32>,
+                           (const void*)conv3x3_fwd<128, 16>, (const void*)conv3x3_fwd<128, 32>})
+      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem) != cudaSuccess) return -3;
+    sm_count[dev].store(sms);
+    attr_set.fetch_or(1ull << dev, std::memory_order_acq_rel);
   }
-  // R image rows of 128 / R columns per CTA: the narrowest tile that covers the width
-  const int R = w > 64 ? 1 : (w > 32 ? 2 : (w > 16 ? 4 : 8));
-  const int W = kTcM / R;
-  const long long segs = (long long)n * ((h + R - 1) / R) * ((w + W - 1) / W);
-  if (segs > 0x7fffffffLL) return -1;
-  const auto* wb = static_cast<const __nv_bfloat16*>(wt_bf16);
+  const int sms = sm_count[dev].load();
+  // rows and pixels of one launch are 32-bit numbers; a larger batch runs in parts
+  const int most = (int)std::max(1LL, std::min<long long>((1LL << 30) / (h + 1), ((1LL << 31) - 1) / ((long long)h * w)));
   cudaStream_t s = (cudaStream_t)stream;
-  const int N = cout % 128 == 0 ? 128 : (cout % 64 == 0 ? 64 : 32);
-  const dim3 grid((unsigned)segs, cout / N);
-  const bool wide = R == 1;
-#define LBM_NN_FWD(NN, WD)                                                                                        \
-  conv3x3_fwd_tc<NN, WD><<<grid, kTcThreads, FwdTcSmem<NN, WD>::bytes(), s>>>(x, wb, bias, y, n, h, w, cin, cout, relu, \
-                                                                              R)
-  if (N == 128) {
-    if (wide) LBM_NN_FWD(128, true); else LBM_NN_FWD(128, false);
-  } else if (N == 64) {
-    if (wide) LBM_NN_FWD(64, true); else LBM_NN_FWD(64, false);
-  } else {
-    if (wide) LBM_NN_FWD(32, true); else LBM_NN_FWD(32, false);
-  }
+  for (int i0 = 0; i0 < n; i0 += most) {
+    const int ni = std::min(most, n - i0);
+    const long long pix = (long long)i0 * h * w;
+    FwdArgs a{x + pix * cin, bias, y + pix * cout, ni, h, w, cin, cout, relu, fwd_plan(ni, h, w, cin, cout, sms)};
+    // tensor map of the weights [tap][cout][cin]: a box holds the nine taps of N output and KC input channels
+    CUtensorMap wmap;
+    if (!weight_map(&wmap, wt_bf16, cin, cout, a.p.N, a.p.KC)) return -3;
+    const unsigned grid = (unsigned)std::min(a.p.items, sms);
+    const int kc16 = a.p.KC == 16;
+#define LBM_NN_FWD(NN)                                                              \
+  do {                                                                              \
+    if (kc16) conv3x3_fwd<NN, 16><<<grid, kCvThreads, a.p.smem, s>>>(a, wmap);      \
+    else conv3x3_fwd<NN, 32><<<grid, kCvThreads, a.p.smem, s>>>(a, wmap);           \
+  } while (0)
+    if (a.p.N == 128) LBM_NN_FWD(128);
+    else if (a.p.N == 64) LBM_NN_FWD(64);
+    else LBM_NN_FWD(32);
 #undef LBM_NN_FWD
-  return status(cudaGetLastError());
+    if (cudaGetLastError() != cudaSuccess) return -3;
+  }
+  return 0;
 }
 
 int lbm_nn_check(void) {
