@@ -49,8 +49,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // image with a zero row between them, so blocks of rows run across image borders.
 //
 // One persistent CTA per SM, three roles that run concurrently:
-//   producers:  look up each staged position's pixel (a table built once per item), load FP32 activations 32 bytes
-//               per thread, round to BF16 into the stage (16-byte stores, free of bank conflicts); one thread starts
+//   producers:  load FP32 activations, 32 bytes per thread, round to BF16 into the stage (16-byte stores, free of bank conflicts); one thread starts
 //               the TMA copy of the stage's weights, [tap][co][KC channels] in the matching 64- or 32-byte swizzle;
 //   products:   one thread issues the tcgen05.mma of a stage and commits them to the barrier that frees it;
 //   epilogue:   reads a finished accumulator (tcgen05.ld), adds the bias, applies the ReLU, transposes through
@@ -61,27 +60,26 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // What bounds it: the wide levels HBM (403 MB for 64 -> 32 on 16 x 256^2: 60 us at copy speed), the deep ones shared
 // memory (an M = 128, K = 16 product reads 4 KB of A, 32 cycles, whatever N) and the pipeline's latency per stage.
 // Measured (GB300, 16 images; the kernel before staged every tile between two CTA barriers, without overlap):
-// 64 -> 32 on 256^2 331 -> 109 us, 128 -> 128 on 64^2 137 -> 31 us, 256 -> 256 on 32^2 101 -> 31 us, one image of the
-// last 54 -> 15 us.  12 producer warps with four 32-byte loads each in flight: 824 us over the network's seventeen
-// forward and data-gradient shapes, against 856 with 8 warps and 830 with 16.
+// 64 -> 32 on 256^2 331 -> 105 us, 128 -> 128 on 64^2 137 -> 33 us, 256 -> 256 on 32^2 101 -> 31 us, one image of the
+// last 54 -> 15 us.  12 producer warps with four 32-byte loads each in flight: 816 us over the network's seventeen
+// forward and data-gradient shapes, against 837 with 8 warps and 827 with 16; loads issued one batch ahead gave
+// nothing, and neither did stores of a lane's own 128-byte line without the transposition (860: slower from 64
+// output channels on).
 // ---------------------------------------------------------------------------
 __device__ unsigned int g_nn_fault = 0;    // set when a bounded wait on the tensor cores gave up
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// shared-memory matrix descriptor: no swizzle, K-major, start / LBO / SBO in bytes
-__device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((addr & 0x3FFFF) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
-         (1ull << 46);
-}
-
-// the same for K-major rows of `row` bytes (32 or 64) in TMA's swizzle of that width, rows contiguous: 8-row groups
-// 8 row bytes apart; a later K = 16 slice of the row starts 32 bytes further
+// Shared-memory matrix descriptors as two words.  Low: start address and leading offset, both in 16 bytes; a later
+// start is an addition (shared memory has fewer than 2^14 units).  High: stride offset, version 1, swizzle.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return (addr >> 4) | ((lbo >> 4) << 16); }
+__device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) { return (sbo >> 4) | (1u << 14); }
+// K-major rows of `row` bytes (32 or 64) in TMA's swizzle of that width, rows contiguous: 8-row groups 8 row bytes
+// apart; a later K = 16 slice of the row starts 32 bytes further
 template <int row>
-__device__ __forceinline__ uint64_t umma_desc_sw(uint32_t addr) {
+__device__ __forceinline__ uint32_t desc_hi_sw() {
   static_assert(row == 32 || row == 64, "swizzle widths used here");
-  return (uint64_t)((addr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)((8 * row) >> 4) << 32) | (1ull << 46) |
-         ((row == 64 ? 4ull : 6ull) << 61);
+  return desc_hi(8 * row) | ((row == 64 ? 4u : 6u) << 29);
 }
 
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both K-major, M x N
@@ -89,17 +87,23 @@ __host__ __device__ constexpr uint32_t umma_idesc(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// D (TMEM) = or += A B^T, one K = 16 product of kind::f16
-__device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+// D (TMEM) = or += A B^T, one K = 16 product of kind::f16, issued by the lane with `leader` set.  The whole warp runs
+// the code around it, so that descriptors stay in uniform registers: with a branch on the lane, the chain of integer
+// instructions of the one thread, not the tensor cores, set the pace of the products.
+__device__ __forceinline__ void umma_f16(uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi, uint32_t idesc,
+                                         uint32_t accumulate, uint32_t leader) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+      "{\n .reg .pred p, q;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n setp.ne.b32 q, %7, 0;\n mov.b64 a, {%1, %2};\n"
+      " mov.b64 b, {%3, %4};\n @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+      "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(leader));
 }
 
-// the products issued so far arrive on an mbarrier when they are done
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar));
+// the products issued so far by the leader arrive on an mbarrier when they are done
+__device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t leader) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+      "r"(leader));
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -109,16 +113,24 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// bounded wait for the completion of phase `parity` of an mbarrier; false when it gave up
+// bounded wait for the completion of phase `parity` of an mbarrier; false when it gave up.  Each poll may suspend the
+// thread for up to 20 us (it wakes when the phase completes), so that waiting warps leave the issue slots to others.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   uint32_t done = 0;
-  for (int it = 0; it < (1 << 24) && !done; ++it)
+  for (int it = 0; it < (1 << 20) && !done; ++it)
     asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(done)
-        : "r"(bar), "r"(parity)
+        : "r"(bar), "r"(parity), "r"(20000)
         : "memory");
   return done != 0;
+}
+
+// eight floats from a 32-byte boundary, through the read-only path
+__device__ __forceinline__ void ldg8(const float* p, float* r) {
+  asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+               : "l"(p));
 }
 
 constexpr int kCvEpi = 8;                          // epilogue warps, two per TMEM lane quarter
@@ -137,6 +149,7 @@ struct FwdPlan {
   int R, T;                  // rows per item, 128-position tiles per item
   int Pn;                    // staged positions allocated per channel group (Pn % 8 == 2: conflict-free stores)
   int stages, stage_bytes, smem, tmem;
+  unsigned mp, mh;           // PosMap's multipliers
   int blocks, items;         // row blocks of the tall image; items = blocks * strips * (cout / N)
 };
 
@@ -148,16 +161,29 @@ struct FwdArgs {
   FwdPlan p;
 };
 
-// barrier of the producer warps with the conjunction of their predicates
-__device__ __forceinline__ bool producers_and(bool ok) {
-  int all;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.and.pred q, 1, %2, p;\n selp.s32 %0, 1, 0, q;\n}\n"
-      : "=r"(all)
-      : "r"((int)ok), "n"(32 * kCvProd)
-      : "memory");
-  return all != 0;
-}
+// Rows and columns of the flat positions of a block, by multiplication: divisions by the pitch and by the rows h + 1
+// of an image of the tall image (exact: the dividends stay below 2^16, or the quotient below 2).
+struct PosMap {
+  unsigned mp, mh;           // ceil(2^32 / pitch), ceil(2^32 / (h + 1)) or 0: a block spans fewer than h + 1 rows
+  int pitch, h, w;
+  int img0, yy0, x0;         // image and row of the block's first row, image column of position column 0
+  __device__ __forceinline__ void block(long long row0, int col0) {
+    img0 = (int)(row0 / (h + 1));
+    yy0 = (int)(row0 - (long long)img0 * (h + 1));
+    x0 = col0;
+  }
+  // pixel of column c of the block's row r, -1 outside the images
+  __device__ __forceinline__ int pixel(int r, int c) const {
+    const int v = yy0 + r;
+    const int k = mh ? (int)__umulhi((unsigned)v, mh) : (v > h ? 1 : 0);
+    const int yy = v - k * (h + 1), xx = x0 + c;
+    return (yy < h && (unsigned)xx < (unsigned)w) ? ((img0 + k) * h + yy) * w + xx : -1;
+  }
+  __device__ __forceinline__ void split(int q, int& r, int& c) const {
+    r = (int)__umulhi((unsigned)q, mp);
+    c = q - r * pitch;
+  }
+};
 
 template <int N, int KC>
 __global__ void __launch_bounds__(kCvThreads, 1)
@@ -166,7 +192,7 @@ __global__ void __launch_bounds__(kCvThreads, 1)
   constexpr int KG = KC / 8;                        // channel groups per stage
   constexpr int kW = 9 * N * KC * 2;                // bytes of a stage's weights
   const FwdPlan& p = a.p;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const int S = p.stages;
   // barriers: activations staged[S], weights landed[S], stage free[S], accumulator ready[2], accumulator free[2]
   const uint32_t b_full = smem_addr(smem), b_w = b_full + 8 * kCvMaxStages, b_empty = b_w + 8 * kCvMaxStages,
@@ -204,26 +230,19 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 
   if (warp > kCvMma) {
     // ---- producers ----
+    PosMap pm{p.mp, p.mh, p.pitch, a.h, a.w};
     const int tp = tid - 32 * (kCvMma + 1);
     constexpr int TP = 32 * kCvProd;
     constexpr int PP = TP / KG;                     // positions per pass of the producer threads
     const int kg = tp % KG, q0 = tp / KG;
-    int* tab = reinterpret_cast<int*>(stage0 + S * p.stage_bytes);   // staged position -> pixel, -1: zero
     int it = 0;                                     // stage count over all items
-    for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
-      // the previous item's table is no longer read; producers leave together when one gave up
-      if (!(ok = producers_and(ok))) break;
+    for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x) {
       const int ct = item % ntile, rest = item / ntile;
-      const int x0 = rest % p.strips * p.Wt, row0 = rest / p.strips * p.R;
+      const int row0 = rest / p.strips * p.R;
       const int NP = (min(p.R, rows_all - row0) + 2) * p.pitch;
-      // the positions' pixels once per item (the same for every channel chunk), shared by the KG threads of a position
-      for (int q = tp; q < NP; q += TP) {
-        const int r = q / p.pitch, xx = x0 - 1 + q - r * p.pitch;
-        const unsigned row = (unsigned)(row0 + r + a.h);      // tall-image row of the halo above, one image further
-        const int img = (int)(row / (unsigned)(a.h + 1)), yy = (int)(row - (unsigned)img * (a.h + 1));
-        tab[q] = (yy < a.h && (unsigned)xx < (unsigned)a.w) ? ((img - 1) * a.h + yy) * a.w + xx : -1;
-      }
-      asm volatile("bar.sync 1, %0;" ::"n"(TP) : "memory");
+      // the halo row above the first image is the zero row of an image before it
+      pm.block(row0 + a.h, rest % p.strips * p.Wt - 1);
+      pm.img0 -= 1;
       for (int s = 0; s < nst; ++s, ++it) {
         const int st = it % S;
         unsigned char* sw = stage0 + st * p.stage_bytes;
@@ -247,7 +266,9 @@ __global__ void __launch_bounds__(kCvThreads, 1)
 #pragma unroll
           for (int u = 0; u < kCvBatch; ++u) {
             const int qq = q + u * PP;
-            const int pix = qq < NP ? tab[qq] : -1;
+            int r, c;
+            pm.split(qq, r, c);
+            const int pix = qq < NP ? pm.pixel(r, c) : -1;
             v[u][0] = v[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (pix >= 0) {
               const float4* at = reinterpret_cast<const float4*>(src + (long long)pix * a.cin);
@@ -270,51 +291,53 @@ __global__ void __launch_bounds__(kCvThreads, 1)
     if (tp == 0)
       for (int k = 0; k < S && k < it; ++k) (void)mbar_wait(b_w + 8 * ((it - 1 - k) % S), (uint32_t)(((it - 1 - k) / S) & 1));
   } else if (warp == kCvMma) {
-    // ---- products: one thread ----
-    if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc(128, N);
-      const uint32_t lbo = (uint32_t)p.Pn * 16;
-      int it = 0, na = 0;
-      for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++na) {
-        const int acc = na & 1;
-        if (na >= 2 && !mbar_wait(b_free + 8 * acc, (uint32_t)((na / 2 - 1) & 1))) {
+    // ---- products: issued by one lane ----
+    constexpr uint32_t idesc = umma_idesc(128, N);
+    const uint32_t leader = lane == 0;
+    const uint32_t ahi = desc_hi(128), bhi = desc_hi_sw<2 * KC>();
+    const uint32_t r1 = (uint32_t)p.pitch, r2 = 2 * r1;
+    int it = 0, na = 0;
+    for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++na) {
+      const int acc = na & 1;
+      if (na >= 2 && !mbar_wait(b_free + 8 * acc, (uint32_t)((na / 2 - 1) & 1))) {
+        ok = false;
+        break;
+      }
+      const int rows = min(p.R, rows_all - item / (ntile * p.strips) * p.R);
+      const int T = ((rows - 1) * p.pitch + p.Wt + 127) / 128;
+      const uint32_t d0 = tmem + (uint32_t)(acc * p.T * N);
+      for (int s = 0; s < nst; ++s, ++it) {
+        const int st = it % S;
+        if (!mbar_wait(b_w + 8 * st, (uint32_t)((it / S) & 1)) || !mbar_wait(b_full + 8 * st, (uint32_t)((it / S) & 1))) {
           ok = false;
           break;
         }
-        const int rows = min(p.R, rows_all - item / (ntile * p.strips) * p.R);
-        const int T = ((rows - 1) * p.pitch + p.Wt + 127) / 128;
-        const uint32_t d0 = tmem + (uint32_t)(acc * p.T * N);
-        for (int s = 0; s < nst; ++s, ++it) {
-          const int st = it % S;
-          if (!mbar_wait(b_w + 8 * st, (uint32_t)((it / S) & 1)) || !mbar_wait(b_full + 8 * st, (uint32_t)((it / S) & 1))) {
-            ok = false;
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          const uint32_t sw = smem_addr(stage0 + st * p.stage_bytes), sx = sw + kW;
-          for (int t = 0; t < T; ++t) {
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint32_t sw = smem_addr(stage0 + st * p.stage_bytes), sx = sw + kW;
+        const uint32_t blo = desc_lo(sw, 16), alo = desc_lo(sx, (uint32_t)p.Pn * 16);
+        for (int t = 0; t < T; ++t) {
 #pragma unroll
-            for (int sub = 0; sub < KC / 16; ++sub) {
-              const uint32_t ax = sx + (uint32_t)(2 * sub * p.Pn + t * 128) * 16;
+          for (int sub = 0; sub < KC / 16; ++sub) {
+            const uint32_t at = alo + (uint32_t)(2 * sub * p.Pn + t * 128);
 #pragma unroll
-              for (int tap = 0; tap < 9; ++tap)
-                umma_f16(d0 + t * N, umma_desc(ax + (uint32_t)((tap / 3) * p.pitch + tap % 3) * 16, lbo, 128),
-                         umma_desc_sw<2 * KC>(sw + tap * N * KC * 2 + 32 * sub), idesc, (s > 0 || sub > 0 || tap > 0) ? 1u : 0u);
-            }
+            for (int tap = 0; tap < 9; ++tap)
+              umma_f16(d0 + t * N, at + (tap < 3 ? 0u : (tap < 6 ? r1 : r2)) + tap % 3, ahi,
+                       blo + (uint32_t)(tap * N * KC * 2 / 16 + 2 * sub), bhi, idesc,
+                       (s > 0 || sub > 0 || tap > 0) ? 1u : 0u, leader);
           }
-          umma_commit(b_empty + 8 * st);
         }
-        if (ok) umma_commit(b_acc + 8 * acc);
+        umma_commit(b_empty + 8 * st, leader);
       }
-      // leave no product in flight: the last commits of the stages
-      for (int k = 0; k < S && k < it; ++k) {
-        const int last = it - 1 - k;
-        (void)mbar_wait(b_empty + 8 * (last % S), (uint32_t)((last / S) & 1));
-      }
+      if (ok) umma_commit(b_acc + 8 * acc, leader);
     }
-    __syncwarp();
+    // leave no product in flight: the last commits of the stages
+    for (int k = 0; k < S && k < it; ++k) {
+      const int last = it - 1 - k;
+      (void)mbar_wait(b_empty + 8 * (last % S), (uint32_t)((last / S) & 1));
+    }
   } else {
     // ---- epilogue ----
+    PosMap pm{p.mp, p.mh, p.pitch, a.h, a.w};
     const int quarter = warp & 3;
     float* buf = tbuf + warp * 1024;                // 32 pixels x 32 channels, 16-byte chunks swizzled by pixel
     const int j = lane & 7;                         // lane j + 8 k stores channels 4 j .. of pixels k, k + 4, ...
@@ -322,9 +345,10 @@ __global__ void __launch_bounds__(kCvThreads, 1)
     for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++na) {
       const int acc = na & 1;
       const int ct = item % ntile, rest = item / ntile;
-      const int x0 = rest % p.strips * p.Wt, row0 = rest / p.strips * p.R;
+      const int row0 = rest / p.strips * p.R;
       const int rows = min(p.R, rows_all - row0);
       const int T = ((rows - 1) * p.pitch + p.Wt + 127) / 128;
+      pm.block(row0, rest % p.strips * p.Wt);
       if (!mbar_wait(b_acc + 8 * acc, (uint32_t)((na / 2) & 1))) {
         ok = false;
         break;
@@ -335,10 +359,9 @@ __global__ void __launch_bounds__(kCvThreads, 1)
         const int t = unit / (N / 32), c0 = unit % (N / 32) * 32;
         // output pixel of this lane's TMEM row, -1: a halo column or row
         const int m = t * 128 + quarter * 32 + lane;
-        const int r = m / p.pitch, c = m - r * p.pitch;
-        const unsigned row = (unsigned)(row0 + r);
-        const int img = (int)(row / (unsigned)(a.h + 1)), yy = (int)(row - (unsigned)img * (a.h + 1));
-        const int pix = (r < rows && yy < a.h && c < p.Wt && x0 + c < a.w) ? (img * a.h + yy) * a.w + x0 + c : -1;
+        int r, c;
+        pm.split(m, r, c);
+        const int pix = (r < rows && c < p.Wt) ? pm.pixel(r, c) : -1;
         const int ch = ct * N + c0 + 4 * j;
         float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
         if (a.bias) bv = make_float4(a.bias[ch], a.bias[ch + 1], a.bias[ch + 2], a.bias[ch + 3]);
@@ -354,9 +377,9 @@ __global__ void __launch_bounds__(kCvThreads, 1)
               : "r"(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((acc * p.T + t) * N + c0)));
           asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<uint4*>(buf + lane * 32 + ((j ^ (lane & 7)) * 4)) =
-                make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+          for (int i = 0; i < 8; ++i)
+            *reinterpret_cast<uint4*>(buf + lane * 32 + ((i ^ (lane & 7)) * 4)) =
+                make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
           __syncwarp();
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
@@ -428,13 +451,15 @@ FwdPlan fwd_plan(int n, int h, int w, int cin, int cout, int sms) {
         p.R = std::min((128 * T - Wt) / pitch + 1, rows_all);
         p.blocks = (rows_all + p.R - 1) / p.R;
         p.R = (rows_all + p.blocks - 1) / p.blocks;
+        p.mp = (unsigned)(((1ull << 32) + pitch - 1) / pitch);
+        p.mh = p.R + 2 <= h ? 0u : (unsigned)(((1ull << 32) + h) / (h + 1));
         p.Pn = 128 * T + 2 * pitch + 2;
         p.Pn += (10 - p.Pn % 8) % 8;                              // Pn % 8 == 2
         p.stage_bytes = (KC / 8) * p.Pn * 16 + 18 * N * KC;
         p.stage_bytes = (p.stage_bytes + 511) / 512 * 512;        // the weights' swizzle pattern repeats every 512 bytes
-        p.stages = std::min(kCvMaxStages, (kCvSmem - kCvHead - 4 * p.Pn) / p.stage_bytes);
+        p.stages = std::min(kCvMaxStages, (kCvSmem - kCvHead) / p.stage_bytes);
         if (p.stages < 2) continue;
-        p.smem = kCvHead + p.stages * p.stage_bytes + 4 * p.Pn;
+        p.smem = kCvHead + p.stages * p.stage_bytes;
         p.tmem = 32;
         while (p.tmem < 2 * T * N) p.tmem *= 2;
         p.items = p.blocks * strips * (cout / N);
@@ -451,385 +476,410 @@ FwdPlan fwd_plan(int n, int h, int w, int cin, int cout, int sms) {
 }
 
 // ---------------------------------------------------------------------------
-// weight gradient on the 5th-generation tensor cores, per chunk z of W-pixel row segments (W = 64, or 32 on
-// images narrower than 64):
-//   part[z][tap][co][ci] = sum_{p in chunk z} dy[p][co] x[p + shift(tap)][ci]
-// A CTA owns 128 output channels x 32 input channels of the three taps (ky, 0..2) of one kernel row ky:
-// D_kx (128 x 32, FP32 in TMEM columns 32 kx ..) += A (128 co x 16 pixels) * B_kx^T (32 ci x 16 pixels),
-// sixteen pixels of the chunk at a time.  The reduction runs over pixels, and both tensors keep their channels
-// innermost, so both operands are staged as BF16 in the canonical MN-major layout without swizzle: core
-// matrices of 8 pixels x 16 bytes (8 channels), the pixels of a segment 16 bytes apart (consecutive core
-// matrices along K 128 bytes apart), the 8-channel groups SBO bytes apart:
-//   A: dy of the segment's W pixels, [co group][pixel];
-//   B: x of image row y + ky - 1 at columns x0 - 1 .. x0 + W, [ci group][column]; tap kx is the window that
-//      starts kx columns (16 kx bytes) further.
-// Channels beyond cout or cin and pixels outside the image are zero.  Two stages as in the forward kernel:
-// a stage is refilled only after the bounded wait for the products that read it.
-// grid (cout tiles of 128, 3 x cin tiles of 32, chunks), 256 threads.
+// weight gradient: dw[ky, kx][co][ci] = sum_p dy[p][co] x[p + shift(ky, kx)][ci]
+//
+// A contraction over the pixels on the tensor cores.  As in the forward kernel, a column strip of Wt columns of the
+// tall image (the batch's images below one another, a zero row between them) is a flat sequence of positions of pitch
+// Wt + 2, and a tap is an offset in it.  With one of the two tensors as U (M side) and the other as V (N side),
+//   D[a, u; b, v] = sum_q U[q + a - 1][u] V[q + (b - 1) pitch][v],   a, b = 0 .. 2,
+// holds all nine taps: U = x: kx = a, ky = 2 - b; U = dy: kx = 2 - a, ky = b.  dy is zero on the halo columns and
+// between the images, so no product counts twice.  Both operands are staged as BF16 in the canonical MN-major layout
+// without swizzle: one plane per 8 channels, 16 bytes per position, so a window of 16 positions (K of one product)
+// may start anywhere.
+//   V: a ring of positions, staged once (halo rows included): tap row b is the window (b - 1) pitch further.  The 16
+//      positions at the start of the ring are stored behind its end too, so that no window wraps.
+//   U: a slot of KP positions per step.  128 channels fill M, one product per a (the window a positions further, the
+//      slot holds one position more on each side).  With at most 64 (32) channels, two (three) of the a share one
+//      product: the slot holds three copies of the channels, shifted by a - 1, and M = 128 covers two (three) of them.
+// The accumulators (one column block of V channels per product and b) stay in TMEM for a segment of positions.
+//
+// A CTA (one per SM) owns a tile of U x V channels and a chunk z of the positions, cut into segments no longer than
+// the float32 chains of the sums should get (and at strip ends); the first segment's sums are written to part[z], the
+// others added.  Producer warps load and round, and sum dy for the bias gradient (unrounded, in a fixed order), in
+// three groups that stage every third step each; one lane issues the products; then four warps move the sums out.
+// An activation or gradient that is not finite makes its whole channel's gradient NaN: the products of the halo
+// columns multiply it by zero.
+//
+// What bounds it: the producers' instructions and load latency on the wide levels (HBM: 40 us for 32 -> 32 on
+// 16 x 256^2), the products elsewhere.  Measured (GB300, 16 images, with the sums and the bias gradient): 32 -> 32 on
+// 256^2 258 -> 116 us, 128 -> 64 on 128^2 393 -> 100 us, 256 -> 128 on 64^2 331 -> 111 us, 256 -> 256 on 32^2 181 -> 80
+// us; the kernels before staged x or dy three times per kernel row between CTA barriers, and dy once more for the bias.
 // ---------------------------------------------------------------------------
-constexpr int kWtM = 128, kWtN = 32, kWtThreads = 256, kWtBatch = 4;
-
-template <int W>
-struct WgTcSmem {
-  static constexpr int kA = (kWtM / 8) * W * 16;
-  static constexpr int kB = (kWtN / 8) * (W + 2) * 16;
-  static constexpr int kStage = kA + kB;
-  static constexpr int bytes() { return 2 * kStage + 64; }
-};
-
 // instruction descriptor of kind::f16 with both operands MN-major (transpose bits 15 and 16)
 __host__ __device__ constexpr uint32_t umma_idesc_mn(int m, int n) { return umma_idesc(m, n) | (1u << 15) | (1u << 16); }
 
-template <int W>
-__global__ void __launch_bounds__(kWtThreads) conv3x3_wgrad_tc(const float* __restrict__ x,
-                                                             const float* __restrict__ dy,
-                                                             float* __restrict__ part, int n, int h, int w,
-                                                             int cin, int cout, long long segs_per_chunk) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  using SM = WgTcSmem<W>;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * SM::kStage);   // one mbarrier per stage
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int co0 = blockIdx.x * kWtM;
-  const int ky = blockIdx.y % 3, ci0 = (blockIdx.y / 3) * kWtN;
-  const int spr = (w + W - 1) / W;                           // segments per image row
-  const long long nseg = (long long)n * h * spr;
-  const long long s0 = (long long)blockIdx.z * segs_per_chunk;
-  const long long s1 = min(nseg, s0 + segs_per_chunk);
-  const int cga = min(kWtM, cout - co0) / 8, cgb = min(kWtN, cin - ci0) / 8;   // channel groups present
-  const uint32_t bar0 = smem_addr(bar);
+constexpr int kWgMaxSlots = 6;
+constexpr int kWgHead = 512;
+constexpr int kWgEpi = 4;                     // warps 0-3: products (one thread of warp 0), then the segment's epilogue
+constexpr int kWgGroups = 3;                  // producer groups of four warps: group g stages steps g, g + 3, ...
+constexpr int kWgGroup = 128, kWgProd = kWgGroups * kWgGroup;
+constexpr int kWgThreads = 32 * kWgEpi + kWgProd;   // 16 warps: 128 registers a thread
+constexpr int kWgBatch = 2;                   // 16-channel groups of each tensor a producer thread has in flight
 
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
-                 "r"(128));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  if (tid == 0) {
-    for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8 * k), "r"(1));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
-  // the channel groups that are not present stay zero in both stages
-  for (int st = 0; st < 2; ++st) {
-    unsigned char* sA = smem + st * SM::kStage;
-    for (int e = tid; e < (kWtM / 8 - cga) * W; e += kWtThreads)
-      *reinterpret_cast<uint4*>(sA + (cga * W + e) * 16) = make_uint4(0u, 0u, 0u, 0u);
-    for (int e = tid; e < (kWtN / 8 - cgb) * (W + 2); e += kWtThreads)
-      *reinterpret_cast<uint4*>(sA + SM::kA + (cgb * (W + 2) + e) * 16) = make_uint4(0u, 0u, 0u, 0u);
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tslot);
-
-  bool ok = true;
-  long long it = 0;
-  for (long long sg = s0; sg < s1; ++sg, ++it) {
-    const int st = (int)(it & 1);
-    unsigned char* sA = smem + st * SM::kStage;
-    unsigned char* sB = sA + SM::kA;
-    // the products of segment it - 2 read this stage: wait for them (phase (it - 2) / 2 of its barrier)
-    if (it >= 2) ok = ok && mbar_wait(bar0 + 8 * st, (uint32_t)(((it - 2) >> 1) & 1));
-    const int img = (int)(sg / ((long long)h * spr));
-    const int y = (int)((sg / spr) % h);
-    const int x0 = (int)(sg % spr) * W;
-    // A: dy of pixels x0 .. x0 + W - 1 of row y, then B: x of row y + ky - 1 at columns x0 - 1 .. x0 + W, in
-    // batches of kWtBatch items per thread whose global loads are all issued before the first conversion and
-    // shared store (a store may not be moved above a later load through pointers that could alias)
-    const int yy = y + ky - 1;
-    const bool row_in = yy >= 0 && yy < h;
-    const int nA = cga * W, nAB = nA + cgb * (W + 2);
-    for (int e0 = 0; e0 < nAB; e0 += kWtBatch * kWtThreads) {
-      float4 pv[kWtBatch], qv[kWtBatch];
-      int off[kWtBatch];   // destination byte offset from sA, -1: none
-#pragma unroll
-      for (int k = 0; k < kWtBatch; ++k) {
-        const int e = e0 + k * kWtThreads + tid;
-        const float* src = nullptr;
-        off[k] = -1;
-        if (e < nA) {
-          const int px = e % W, cg = e / W;
-          const int xc = x0 + px;
-          if (xc < w) src = dy + (((long long)img * h + y) * w + xc) * cout + co0 + 8 * cg;
-          off[k] = (cg * W + px) * 16;
-        } else if (e < nAB) {
-          const int j = (e - nA) % (W + 2), cg = (e - nA) / (W + 2);
-          const int xc = x0 + j - 1;
-          if (row_in && xc >= 0 && xc < w) src = x + (((long long)img * h + yy) * w + xc) * cin + ci0 + 8 * cg;
-          off[k] = SM::kA + (cg * (W + 2) + j) * 16;
-        }
-        pv[k] = qv[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (src) {
-          pv[k] = __ldg(reinterpret_cast<const float4*>(src));
-          qv[k] = __ldg(reinterpret_cast<const float4*>(src + 4));
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < kWtBatch; ++k)
-        if (off[k] >= 0)
-          *reinterpret_cast<uint4*>(sA + off[k]) =
-              make_uint4(pack_bf16(pv[k].x, pv[k].y), pack_bf16(pv[k].z, pv[k].w), pack_bf16(qv[k].x, qv[k].y),
-                         pack_bf16(qv[k].z, qv[k].w));
-    }
-    asm volatile("fence.proxy.async.shared::cta;");       // generic-proxy stores visible to the tensor cores
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (tid == 0 && ok) {
-      constexpr uint32_t idesc = umma_idesc_mn(kWtM, kWtN);
-#pragma unroll 1
-      for (int kx = 0; kx < 3; ++kx) {
-#pragma unroll
-        for (int ks = 0; ks < W / 16; ++ks) {
-          // MN-major, no swizzle: LBO = stride of core matrices along K, SBO = along M / N
-          const uint64_t ad = umma_desc(smem_addr(sA + ks * 256), 128, W * 16);
-          const uint64_t bd = umma_desc(smem_addr(sB + (kx + 16 * ks) * 16), 128, (W + 2) * 16);
-          const uint32_t acc = (it > 0 || ks > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + 32u * kx),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-        }
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 8 * st));
-    }
-  }
-  // the last commit completes after every product issued before it
-  if (it > 0) ok = ok && mbar_wait(bar0 + 8 * (int)((it - 1) & 1), (uint32_t)(((it - 1) >> 1) & 1));
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (ok) {
-    // warps w and w + 4 read TMEM lanes 32 (w % 4) .. + 31 (= output channels); of the six 16-column blocks
-    // (kx = block / 2) warps 0-3 take the first three, warps 4-7 the others
-    const int q = warp & 3;
-    const int co = co0 + q * 32 + lane;
-#pragma unroll 1
-    for (int blk = 3 * (warp >> 2); blk < 3 * (warp >> 2) + 3; ++blk) {
-      const int kx = blk >> 1, c0 = (blk & 1) * 16;
-      uint32_t r[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-          "%14, %15}, [%16];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(32 * kx + c0)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;");
-      if (co < cout && c0 < cgb * 8) {
-        float* dst = part + (((long long)blockIdx.z * 9 + 3 * ky + kx) * cout + co) * cin + ci0 + c0;
-#pragma unroll
-        for (int j = 0; j < 16; j += 4) {
-          const float4 o = it > 0 ? make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                                __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]))
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-          *reinterpret_cast<float4*>(dst + j) = o;
-        }
-      }
-    }
-  } else if (tid == 0) {
-    atomicExch(&g_nn_fault, 1u);
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
+// barrier `id` of `count` threads with the conjunction of their predicates
+template <int id, int count>
+__device__ __forceinline__ bool meet(bool ok) {
+  int all;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.s32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+      : "=r"(all)
+      : "r"((int)ok), "n"(id), "n"(count)
+      : "memory");
+  return all != 0;
 }
 
-// ---------------------------------------------------------------------------
-// weight gradient for at most 64 output channels: the three kernel rows folded into the 128 rows of M, 32
-// output channels per CTA.
-// With q = p + shift(tap), part[z][tap][co][ci] = sum_q dy[q - shift(tap)][co] x[q][ci]: for a segment of W
-// pixels q of row y, B is x of those pixels (32 input channels, unshifted) and A row (ky, co), 32 ky + co, is dy
-// of image row y - ky + 1, so one product per column offset kx covers the three kernel rows:
-// D_kx (128 x 32, rows 96 .. 127 zero, TMEM columns 32 kx ..) += A_kx (128 x 16 pixels) * B^T (32 x 16 pixels).
-// Both operands are BF16 in the canonical MN-major layout without swizzle, as in conv3x3_wgrad_tc:
-//   A: [ky][co group][column] for columns x0 - 1 .. x0 + W of dy rows y + 1, y, y - 1; the window of kx starts
-//      2 - kx columns (16 (2 - kx) bytes) in;
-//   B: [ci group][pixel] for pixels x0 .. x0 + W - 1 of x row y.
-// grid (cout tiles of 32, cin tiles of 32, chunks), 256 threads, two stages.
-// ---------------------------------------------------------------------------
-template <int W>
-struct WgRowsSmem {
-  static constexpr int kA = (kWtM / 8) * (W + 2) * 16;
-  static constexpr int kB = (kWtN / 8) * W * 16;
-  static constexpr int kStage = kA + kB;
-  static constexpr int bytes() { return 2 * kStage + 64; }
+struct WgradPlan {
+  int u_dy;                    // 1: U = dy, V = x; 0: U = x, V = dy
+  int mt, vt, mb;              // channels of U and V per tile; products per b (3 without folding, 2, 1)
+  int utiles, vtiles;
+  int Wt, pitch, strips;
+  int KP, slots;               // positions per step, steps in flight
+  int ulen, rv, vlen;          // plane lengths: U slot; V ring, V plane (ring + 16, padded)
+  int u_bytes, v_bytes, smem, tmem;
+  int seg_steps;               // longest segment
+  unsigned mp, mh;
+  long long len, steps;        // positions and steps of a strip
+  long long chunks;            // partial sums
+  long long bias_chunks, ws_chunks;
 };
 
-template <int W>
-__global__ void __launch_bounds__(kWtThreads) conv3x3_wgrad_tc_rows(const float* __restrict__ x,
-                                                                  const float* __restrict__ dy,
-                                                                  float* __restrict__ part, int n, int h, int w,
-                                                                  int cin, int cout, long long segs_per_chunk) {
+struct WgradArgs {
+  const float *u, *v;
+  float *part, *bias_part;     // bias_part: [chunks][cout] or NULL
+  int n, h, w, cu, cv, cin, cout;
+  int wide;                    // both tensors on 32 bytes: 32-byte loads
+  WgradPlan p;
+};
+
+// MB: products per b (1: three copies of U in one, 2: two and one, 3: no copies)
+template <int MB>
+__global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  using SM = WgRowsSmem<W>;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + 2 * SM::kStage);   // one mbarrier per stage
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bar + 2);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int co0 = blockIdx.x * 32, ci0 = blockIdx.y * kWtN;
-  const int spr = (w + W - 1) / W;                           // segments per image row
-  const long long nseg = (long long)n * h * spr;
-  const long long s0 = (long long)blockIdx.z * segs_per_chunk;
-  const long long s1 = min(nseg, s0 + segs_per_chunk);
-  const int cga = min(32, cout - co0) / 8, cgb = min(kWtN, cin - ci0) / 8;   // channel groups present
-  const uint32_t bar0 = smem_addr(bar);
+  const WgradPlan& p = a.p;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int S = p.slots;
+  // barriers: step staged[S], step free[S], accumulator ready
+  const uint32_t b_full = smem_addr(smem), b_empty = b_full + 8 * kWgMaxSlots, b_acc = b_empty + 8 * kWgMaxSlots;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + 16 * kWgMaxSlots + 8);
+  unsigned char* const su = smem + kWgHead;                  // U slots, then the V ring
+  unsigned char* const sv = su + (size_t)S * p.u_bytes;
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
-                 "r"(128));
+                 "r"(p.tmem));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int k = 0; k < 2; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar0 + 8 * k), "r"(1));
+    for (int k = 0; k < S; ++k) {
+      mbar_init(b_full + 8 * k, kWgGroup);
+      mbar_init(b_empty + 8 * k, 1);
+    }
+    mbar_init(b_acc, 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
-  // both stages start zero: the channel groups that are not present, and rows 96 .. 127 of A, stay so
-  for (int e = tid; e < 2 * SM::kStage / 16; e += kWtThreads)
-    *reinterpret_cast<uint4*>(smem + 16 * e) = make_uint4(0u, 0u, 0u, 0u);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tslot);
 
+  const int ntile = p.utiles * p.vtiles;
+  const int tile = blockIdx.x % ntile;
+  const long long z = blockIdx.x / ntile;
+  const int u0 = tile % p.utiles * p.mt, v0 = tile / p.utiles * p.vt;
+  const int nu = min(p.mt, a.cu - u0), nv = min(p.vt, a.cv - v0);   // channels present (multiples of 16)
+  const long long total = p.steps * p.strips;
+  const long long t0 = total * z / p.chunks, t1 = total * (z + 1) / p.chunks;   // steps of this chunk
+  // end of the segment that starts at step t
+  auto seg_end = [&](long long t) {
+    return min(min(t1, t + p.seg_steps), (t / p.steps + 1) * p.steps);
+  };
   bool ok = true;
-  long long it = 0;
-  for (long long sg = s0; sg < s1; ++sg, ++it) {
-    const int st = (int)(it & 1);
-    unsigned char* sA = smem + st * SM::kStage;
-    // the products of segment it - 2 read this stage: wait for them (phase (it - 2) / 2 of its barrier)
-    if (it >= 2) ok = ok && mbar_wait(bar0 + 8 * st, (uint32_t)(((it - 2) >> 1) & 1));
-    const int img = (int)(sg / ((long long)h * spr));
-    const int y = (int)((sg / spr) % h);
-    const int x0 = (int)(sg % spr) * W;
-    // A: dy rows y + 1, y, y - 1 (ky = 0, 1, 2) at columns x0 - 1 .. x0 + W; then B: x row y at x0 .. x0 + W - 1.
-    // The global loads of kWtBatch items per thread are issued before their conversions and shared stores.
-    const int nA = 3 * cga * (W + 2), nAB = nA + cgb * W;
-    for (int e0 = 0; e0 < nAB; e0 += kWtBatch * kWtThreads) {
-      float4 pv[kWtBatch], qv[kWtBatch];
-      int off[kWtBatch];   // destination byte offset from sA, -1: none
+
+  if (warp >= kWgEpi) {
+    // ---- producers ----
+    const int tp = tid - 32 * kWgEpi, tg = tp % kWgGroup, group = tp / kWgGroup;
+    PosMap pm{p.mp, p.mh, p.pitch, a.h, a.w};
+    auto pow2 = [](int g) { return g <= 1 ? 1 : (g <= 2 ? 2 : (g <= 4 ? 4 : 8)); };
+    // thread -> (position, 16-channel group), groups fastest; a thread keeps its group for the whole chunk
+    const int gu = pow2(nu / 16), gv = pow2(nv / 16);
+    const int ku = tg % gu, qu = tg / gu, kv = tg % gv, qv = tg / gv;
+    const int pu = kWgGroup / gu, pv = kWgGroup / gv;        // positions per pass of a group
+    const bool u_on = ku < nu / 16, v_on = kv < nv / 16;
+    const bool bias = a.bias_part != nullptr && (p.u_dy ? v0 == 0 : u0 == 0);
+    float bs[16];
 #pragma unroll
-      for (int k = 0; k < kWtBatch; ++k) {
-        const int e = e0 + k * kWtThreads + tid;
-        const float* src = nullptr;
-        off[k] = -1;
-        if (e < nA) {
-          const int j = e % (W + 2), cg = (e / (W + 2)) % cga, ky = e / ((W + 2) * cga);
-          const int yy = y - ky + 1, xc = x0 + j - 1;
-          if (yy >= 0 && yy < h && xc >= 0 && xc < w)
-            src = dy + (((long long)img * h + yy) * w + xc) * cout + co0 + 8 * cg;
-          off[k] = ((ky * 4 + cg) * (W + 2) + j) * 16;
-        } else if (e < nAB) {
-          const int j = (e - nA) % W, cg = (e - nA) / W;
-          const int xc = x0 + j;
-          if (xc < w) src = x + (((long long)img * h + y) * w + xc) * cin + ci0 + 8 * cg;
-          off[k] = SM::kA + (cg * W + j) * 16;
-        }
-        pv[k] = qv[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (src) {
-          pv[k] = __ldg(reinterpret_cast<const float4*>(src));
-          qv[k] = __ldg(reinterpret_cast<const float4*>(src + 4));
-        }
-      }
+    for (int k = 0; k < 16; ++k) bs[k] = 0.f;
+    const float* usrc = a.u + u0 + 16 * ku;
+    const float* vsrc = a.v + v0 + 16 * kv;
+    // positions are counted from the segment's first; those in [lo, hi) lie in the strip, `off` past the map's row 0
+    int lo = 0, hi = 0, off = 0;
+    // sixteen channels of position q, zero outside the images; dy only on the strip's own columns
+    auto fetch = [&](float (&r)[16], const float* src, int c, bool dy, int q, bool on) {
 #pragma unroll
-      for (int k = 0; k < kWtBatch; ++k)
-        if (off[k] >= 0)
-          *reinterpret_cast<uint4*>(sA + off[k]) =
-              make_uint4(pack_bf16(pv[k].x, pv[k].y), pack_bf16(pv[k].z, pv[k].w), pack_bf16(qv[k].x, qv[k].y),
-                         pack_bf16(qv[k].z, qv[k].w));
-    }
-    asm volatile("fence.proxy.async.shared::cta;");       // generic-proxy stores visible to the tensor cores
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (tid == 0 && ok) {
-      constexpr uint32_t idesc = umma_idesc_mn(kWtM, kWtN);
-#pragma unroll 1
-      for (int kx = 0; kx < 3; ++kx) {
+      for (int k = 0; k < 16; ++k) r[k] = 0.f;
+      if (on && q >= lo && q < hi) {
+        int row, col;
+        pm.split(q + off, row, col);
+        const int pix = pm.pixel(row, col);
+        if (pix >= 0 && (!dy || (unsigned)(col - 1) < (unsigned)p.Wt)) {
+          const float* at = src + (long long)pix * c;
+          if (a.wide) {
+            ldg8(at, r);
+            ldg8(at + 8, r + 8);
+          } else {
 #pragma unroll
-        for (int ks = 0; ks < W / 16; ++ks) {
-          const uint64_t ad = umma_desc(smem_addr(sA + (2 - kx + 16 * ks) * 16), 128, (W + 2) * 16);
-          const uint64_t bd = umma_desc(smem_addr(sA + SM::kA + ks * 256), 128, W * 16);
-          const uint32_t acc = (it > 0 || ks > 0) ? 1u : 0u;
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + 32u * kx),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+            for (int k = 0; k < 16; k += 4) {
+              const float4 t = __ldg(reinterpret_cast<const float4*>(at + k));
+              r[k] = t.x, r[k + 1] = t.y, r[k + 2] = t.z, r[k + 3] = t.w;
+            }
+          }
         }
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar0 + 8 * st));
+    };
+    auto round8 = [](const float* r) {
+      return make_uint4(pack_bf16(r[0], r[1]), pack_bf16(r[2], r[3]), pack_bf16(r[4], r[5]), pack_bf16(r[6], r[7]));
+    };
+    auto tally = [&](const float (&r)[16]) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) bs[k] += r[k];
+    };
+    int qb = 0;                                              // end of the segment
+    auto put_v = [&](const float (&r)[16], int q, int at) {
+      if (at >= p.rv) at -= p.rv;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const uint4 val = round8(r + 8 * e);
+        unsigned char* dst = sv + ((2 * kv + e) * p.vlen + at) * 16;
+        *reinterpret_cast<uint4*>(dst) = val;
+        if (at < 16) *reinterpret_cast<uint4*>(dst + p.rv * 16) = val;
+      }
+      if (bias && !p.u_dy && q >= 0 && q < qb) tally(r);
+    };
+    auto put_u = [&](const float (&r)[16], unsigned char* slot, int at) {   // at: position - (first - 1)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const uint4 val = round8(r + 8 * e);
+        unsigned char* dst = slot + ((2 * ku + e) * p.ulen + at) * 16;
+        if (MB == 3) {
+          *reinterpret_cast<uint4*>(dst) = val;
+        } else {
+          // copy c holds position first + i + c - 1 at i
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            if ((unsigned)(at - c) < (unsigned)p.KP)
+              *reinterpret_cast<uint4*>(dst + (c * ((MB == 1 ? 4 : 8) * p.ulen) - c) * 16) = val;
+        }
+      }
+      if (bias && p.u_dy && at >= 1 && at <= p.KP) tally(r);
+    };
+    int it = 0;                                              // steps over all segments
+    for (long long t = t0; t < t1;) {
+      const long long te = seg_end(t);
+      const int strip = (int)(t / p.steps);
+      const long long first = t % p.steps * p.KP, row0 = first / p.pitch - 2;
+      qb = (int)(te - t) * p.KP;
+      // map of the segment: from the row two above its first position's (tall-image rows shifted by two images)
+      pm.block(row0 + 2LL * (a.h + 1), strip * p.Wt - 1);
+      pm.img0 -= 2;
+      off = (int)(first - row0 * p.pitch);
+      lo = (int)max(-first, -(1LL << 30));
+      hi = (int)min(p.len - first, 1LL << 30);
+      // the ring restarts at position -pitch: every step of the previous segment is staged (the groups meet first: a
+      // phase may only be waited for once the one before it is known to be complete) and its products are done; then
+      // the ring's first 2 pitch positions, by all producers
+      if (!(ok = meet<1, kWgProd>(ok))) break;
+      for (int k = 1; k <= S && k <= it && ok; ++k)
+        ok = mbar_wait(b_empty + 8 * ((it - k) % S), (uint32_t)(((it - k) / S) & 1));
+      if (ok)
+        for (int q = group * pv + qv; q < 2 * p.pitch; q += kWgGroups * pv * kWgBatch) {
+          float r[kWgBatch][16];
+#pragma unroll
+          for (int k = 0; k < kWgBatch; ++k) {
+            const int at = q + k * kWgGroups * pv;
+            fetch(r[k], vsrc, a.cv, !p.u_dy, at - p.pitch, v_on && at < 2 * p.pitch);
+          }
+#pragma unroll
+          for (int k = 0; k < kWgBatch; ++k) {
+            const int at = q + k * kWgGroups * pv;
+            if (v_on && at < 2 * p.pitch) put_v(r[k], at - p.pitch, at);
+          }
+        }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      if (!(ok = meet<1, kWgProd>(ok))) break;
+      const int nstep = (int)(te - t);
+      const int base = it;
+      for (int sn = (group + kWgGroups - base % kWgGroups) % kWgGroups; sn < nstep; sn += kWgGroups) {
+        const int step = base + sn, st = step % S, qs = sn * p.KP;
+        if (step >= S && !mbar_wait(b_empty + 8 * st, (uint32_t)((step / S - 1) & 1))) {
+          ok = false;
+          break;
+        }
+        const int ring = (2 * p.pitch + qs) % p.rv;          // ring index of position qs + pitch
+        unsigned char* slot = su + (size_t)st * p.u_bytes;
+        for (int iv = qv, iu = qu; iv < p.KP || iu < p.KP + 2; iv += kWgBatch * pv, iu += kWgBatch * pu) {
+          float rv[kWgBatch][16], ru[kWgBatch][16];
+#pragma unroll
+          for (int k = 0; k < kWgBatch; ++k)
+            fetch(rv[k], vsrc, a.cv, !p.u_dy, qs + p.pitch + iv + k * pv, v_on && iv + k * pv < p.KP);
+#pragma unroll
+          for (int k = 0; k < kWgBatch; ++k)
+            fetch(ru[k], usrc, a.cu, p.u_dy, qs - 1 + iu + k * pu, u_on && iu + k * pu < p.KP + 2);
+#pragma unroll
+          for (int k = 0; k < kWgBatch; ++k)
+            if (v_on && iv + k * pv < p.KP) put_v(rv[k], qs + p.pitch + iv + k * pv, ring + iv + k * pv);
+#pragma unroll
+          for (int k = 0; k < kWgBatch; ++k)
+            if (u_on && iu + k * pu < p.KP + 2) put_u(ru[k], slot, iu + k * pu);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive(b_full + 8 * st);
+      }
+      it = base + nstep;
+      t = te;
     }
+    ok = meet<1, kWgProd>(ok);
+    // bias partials: the threads of a channel group in their order.  The stages are free once the products are done.
+    for (int k = 1; k <= S && k <= it && ok; ++k)
+      ok = mbar_wait(b_empty + 8 * ((it - k) % S), (uint32_t)(((it - k) / S) & 1));
+    if (bias) {
+      const int g = p.u_dy ? gu : gv, nc = p.u_dy ? nu : nv, c0 = p.u_dy ? u0 : v0;
+      float* red = reinterpret_cast<float*>(sv);             // [16][kWgProd]: fits the ring (at least 24.6 KB)
+      if (ok) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) red[k * kWgProd + tp] = bs[k];
+      }
+      (void)meet<1, kWgProd>(ok);
+      if (tp < nc) {
+        float s = 0.f;
+        for (int k = tp / 16; k < kWgProd; k += g) s += red[(tp & 15) * kWgProd + k];
+        a.bias_part[z * a.cout + c0 + tp] = s;
+      }
+    }
+  } else {
+    // ---- products: one thread; then the epilogue of the segment: four warps ----
+    const uint32_t idesc = umma_idesc_mn(128, nv);
+    const uint32_t usbo = (uint32_t)p.ulen * 16, vsbo = (uint32_t)p.vlen * 16;
+    const uint32_t ahi = desc_hi(usbo), bhi = desc_hi(vsbo);
+    const uint32_t vlo = desc_lo(smem_addr(sv), 128), ulo = desc_lo(smem_addr(su), 128);
+    const uint32_t leader = lane == 0;
+    const int quarter = warp;
+    const int fold = MB == 3 ? 1 : (MB == 2 ? 2 : 4);    // copies of U's channels in one product's 128 rows
+    const int row = quarter * 32 + lane;
+    const int per = 128 / fold;                              // rows per copy
+    const int c = row % per;                                 // U channel of this lane's TMEM row
+    int it = 0, ns = 0;
+    for (long long t = t0; t < t1 && ok; ++ns) {
+      const long long te = seg_end(t);
+      if (warp == 0) {
+        // ring indices of the windows of tap rows 0 .. 2 at the segment's first position
+        int r0 = 0, r1 = p.pitch, r2 = 2 * p.pitch;
+        for (long long s = t; s < te; ++s, ++it) {
+          const int st = it % S;
+          if (!mbar_wait(b_full + 8 * st, (uint32_t)((it / S) & 1))) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t slot = ulo + (uint32_t)(st * (p.u_bytes / 16));
+          for (int k = 0; k < p.KP; k += 16) {
+            const uint32_t acc = (s > t || k > 0) ? 1u : 0u;
+            const uint32_t w0 = vlo + (uint32_t)r0, w1 = vlo + (uint32_t)r1, w2 = vlo + (uint32_t)r2;
+            for (int m = 0; m < MB; ++m) {
+              // mb 3: the window m positions further; else block m of the copies' planes
+              const uint32_t ua = slot + (uint32_t)k + (uint32_t)(MB == 3 ? m : m * 16 * p.ulen);
+              const uint32_t d = tmem + (uint32_t)(m * 3 * p.vt);
+              umma_f16(d, ua, ahi, w0, bhi, idesc, acc, leader);
+              umma_f16(d + p.vt, ua, ahi, w1, bhi, idesc, acc, leader);
+              umma_f16(d + 2 * p.vt, ua, ahi, w2, bhi, idesc, acc, leader);
+            }
+            r0 = r0 + 16 >= p.rv ? r0 + 16 - p.rv : r0 + 16;
+            r1 = r1 + 16 >= p.rv ? r1 + 16 - p.rv : r1 + 16;
+            r2 = r2 + 16 >= p.rv ? r2 + 16 - p.rv : r2 + 16;
+          }
+          umma_commit(b_empty + 8 * st, leader);
+        }
+        if (ok) umma_commit(b_acc, leader);
+        __syncwarp();
+      }
+      ok = mbar_wait(b_acc, (uint32_t)(ns & 1)) && ok;
+      if (!(ok = meet<2, 32 * kWgEpi>(ok))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      const int nblk = nv / 16;
+      for (int unit = 0; unit < MB * 3 * nblk; ++unit) {
+        const int blk = unit % nblk, b = unit / nblk % 3, m = unit / (3 * nblk);
+        const int cp = m * fold + row / per;                 // a of this row
+        uint32_t r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+            "%15}, [%16];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+            : "r"(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((m * 3 + b) * p.vt + blk * 16)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;");
+        if (cp < 3 && c < nu) {
+          const int tap = p.u_dy ? 3 * b + 2 - cp : 3 * (2 - b) + cp;
+          float* base = a.part + (z * 9 + tap) * a.cout * a.cin;
+          if (p.u_dy) {                                      // row = co, columns = ci
+            float4* dst = reinterpret_cast<float4*>(base + (long long)(u0 + c) * a.cin + v0 + blk * 16);
+            float4 e[4];                                     // the earlier segments' sums, all loads before the stores
+#pragma unroll
+            for (int j = 0; j < 4; ++j) e[j] = ns > 0 ? dst[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              dst[j] = make_float4(e[j].x + __uint_as_float(r[4 * j]), e[j].y + __uint_as_float(r[4 * j + 1]),
+                                   e[j].z + __uint_as_float(r[4 * j + 2]), e[j].w + __uint_as_float(r[4 * j + 3]));
+          } else {                                           // row = ci, columns = co
+            float* dst = base + (long long)(v0 + blk * 16) * a.cin + u0 + c;
+            float e[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) e[j] = ns > 0 ? dst[(long long)j * a.cin] : 0.f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) dst[(long long)j * a.cin] = e[j] + __uint_as_float(r[j]);
+          }
+        }
+      }
+      // the sums are read before the next segment overwrites them
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      (void)meet<2, 32 * kWgEpi>(true);
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      t = te;
+    }
+    if (warp == 0)
+      for (int k = 1; k <= S && k <= it; ++k)                // leave no product in flight
+        (void)mbar_wait(b_empty + 8 * ((it - k) % S), (uint32_t)(((it - k) / S) & 1));
   }
-  // the last commit completes after every product issued before it
-  if (it > 0) ok = ok && mbar_wait(bar0 + 8 * (int)((it - 1) & 1), (uint32_t)(((it - 1) >> 1) & 1));
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (ok) {
-    // warps w and w + 4 read TMEM lanes 32 (w % 4) .. + 31 = (ky = w % 4, co); lanes 96 .. 127 are the zero rows.
-    // Of the six 16-column blocks (kx = block / 2) warps 0-3 take the first three, warps 4-7 the others.
-    const int ky = warp & 3, co = co0 + lane;
-#pragma unroll 1
-    for (int blk = 3 * (warp >> 2); blk < 3 * (warp >> 2) + 3; ++blk) {
-      const int kx = blk >> 1, c0 = (blk & 1) * 16;
-      uint32_t r[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-          "%14, %15}, [%16];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(tmem + ((uint32_t)(ky * 32) << 16) + (uint32_t)(32 * kx + c0)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;");
-      if (ky < 3 && co < cout && c0 < cgb * 8) {
-        float* dst = part + (((long long)blockIdx.z * 9 + 3 * ky + kx) * cout + co) * cin + ci0 + c0;
-#pragma unroll
-        for (int j = 0; j < 16; j += 4) {
-          const float4 o = it > 0 ? make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]),
-                                                __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]))
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-          *reinterpret_cast<float4*>(dst + j) = o;
-        }
-      }
-    }
-  } else if (tid == 0) {
-    atomicExch(&g_nn_fault, 1u);
-  }
+  if (!ok) atomicExch(&g_nn_fault, 1u);
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(128));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(p.tmem));
 }
 
-// out[i] = sum_z part[z][i]: 8 lanes per output take the chunks z = lane, lane + 8, ... in order, then the 8 lane
-// sums are added in a fixed tree (deterministic).  Block = 32 outputs x 8 lanes.
-__global__ void __launch_bounds__(256) sum_parts(const float* __restrict__ part, float* __restrict__ out, long long n,
-                                                 int chunks) {
-  __shared__ float red[8][32];
-  const int o = threadIdx.x & 31, lane = threadIdx.x >> 5;
-  const long long i = (long long)blockIdx.x * 32 + o;
+// out[i] = sum_z part[z][i] for the n weight gradients and, in the blocks behind theirs, for the n2 bias gradients: L
+// lanes per output take the chunks z = lane, lane + L, ... in order, then the lane sums are added in a fixed tree
+// (deterministic).  Block = 32 outputs x L lanes.  A few MB out of L2, bound by latency: about ten loads per lane (152
+// chunks of 32 x 32 channels: 7.5 + 6.6 us as two launches of eight lanes, 5 us as this one of sixteen).
+constexpr int kSumLanes = 16;   // most lanes
+__global__ void __launch_bounds__(32 * kSumLanes) sum_parts(const float* __restrict__ part, float* __restrict__ out,
+                                                            long long n, const float* __restrict__ part2,
+                                                            float* __restrict__ out2, int n2, int chunks) {
+  __shared__ float red[kSumLanes][32];
+  const long long nb = (n + 31) / 32;
+  long long blk = blockIdx.x;
+  if (blk >= nb) part = part2, out = out2, n = n2, blk -= nb;
+  const int o = threadIdx.x & 31, lane = threadIdx.x >> 5, L = blockDim.x >> 5;
+  const long long i = blk * 32 + o;
   float s = 0.f;
   if (i < n) {
-#pragma unroll 4
-    for (int z = lane; z < chunks; z += 8) s += part[(long long)z * n + i];
+#pragma unroll 10
+    for (int z = lane; z < chunks; z += L) s += part[(long long)z * n + i];
   }
   red[lane][o] = s;
   __syncthreads();
-  if (lane == 0 && i < n)
-    out[i] = ((red[0][o] + red[1][o]) + (red[2][o] + red[3][o])) + ((red[4][o] + red[5][o]) + (red[6][o] + red[7][o]));
-}
-
-// bias gradient partials: part[z][c] = sum_{p in chunk z} dy[p][c]; block = 32 channels x 8 pixel lanes,
-// lanes combined in a fixed order (deterministic).  grid (ceil(c / 32), chunks)
-__global__ void __launch_bounds__(256) colsum_part(const float* __restrict__ dy, float* __restrict__ part, long long P,
-                                                   int c, long long chunk) {
-  __shared__ float red[8][32];
-  const int ch = blockIdx.x * 32 + (threadIdx.x & 31), r = threadIdx.x >> 5;
-  const long long pb = (long long)blockIdx.y * chunk, pe = min(P, pb + chunk);
-  float s = 0.f;
-  if (ch < c) {
-#pragma unroll 8
-    for (long long p = pb + r; p < pe; p += 8) s += dy[p * c + ch];
+  for (int k = L / 2; k > 0; k >>= 1) {
+    if (lane < k) red[lane][o] += red[lane + k][o];
+    __syncthreads();
   }
-  red[r][threadIdx.x & 31] = s;
-  __syncthreads();
-  if (r == 0 && ch < c) {
-    float v = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v += red[k][threadIdx.x & 31];
-    part[(long long)blockIdx.y * c + ch] = v;
-  }
+  if (lane == 0 && i < n) out[i] = red[0][o];
 }
 
 // wt'[tap][ci][co] = wt[8 - tap][co][ci]: the kernel of the data gradient
@@ -1145,26 +1195,86 @@ namespace {
 
 constexpr long long kBiasChunk = 4096;
 
-// row segments per CTA of the weight gradient: at most four CTAs per SM (the TMEM of 4 x 128 columns) over the
-// (co, ky, ci) tiles, so that every CTA is resident in one wave
-struct WgradPlan {
-  int W;
-  long long segs, per_chunk, chunks, bias_chunks, tiles;
-};
-
+// Tiles and chunks of the weight gradient: the orientation, channel tiles and step length with the least modelled time,
+// (positions per chunk) x the larger of the staging time (12 bytes per SM and cycle, measured for the producer warps)
+// and the product time (shared-memory reads: 32 cycles of U, vt / 4 of V per product).  One CTA per SM, one wave.
+// The workspace keeps at most four sets of partial sums per SM's share of 32 x 32 (up to 64 output channels) or 128 x
+// 32 x one kernel row channel tiles; one set of them is the bias partials' room.
 WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
-  WgradPlan p;
-  p.W = w >= 64 ? 64 : 32;
-  p.segs = (long long)n * h * ((w + p.W - 1) / p.W);
-  // at most 64 output channels: the kernel rows folded into M (a CTA per 32 x 32 channel tile); else a CTA per
-  // kernel row and 128 x 32 tile
-  p.tiles = cout <= 64 ? (long long)((cout + 31) / 32) * ((cin + kWtN - 1) / kWtN)
-                       : (long long)((cout + kWtM - 1) / kWtM) * 3 * ((cin + kWtN - 1) / kWtN);
-  const long long want = std::max(1LL, (4LL * 152) / p.tiles);
-  p.per_chunk = std::max(1LL, (p.segs + want - 1) / want);
-  p.chunks = (p.segs + p.per_chunk - 1) / p.per_chunk;
-  p.bias_chunks = ((long long)n * h * w + kBiasChunk - 1) / kBiasChunk;
-  return p;
+  constexpr int sms = 152;
+  const int old_tiles = cout <= 64 ? ((cout + 31) / 32) * ((cin + 31) / 32) : ((cout + 127) / 128) * 3 * ((cin + 31) / 32);
+  const long long most = std::max(1LL, 4LL * sms / old_tiles - 1);
+  // longest float32 chain of one accumulator: the pixels over the partial sums that fit the workspace
+  const long long pixels = (long long)n * h * w;
+  const long long chain = std::max(256LL, pixels * old_tiles / (4 * sms));
+  WgradPlan best{};
+  double best_cost = -1.0;
+  for (int u_dy = 0; u_dy < 2; ++u_dy) {
+    const int cu = u_dy ? cout : cin, cv = u_dy ? cin : cout;
+    for (int mt = 32; mt <= 128; mt *= 2) {
+      if (mt > 32 && cu <= mt / 2) break;
+      const int mb = mt / 32 > 2 ? 3 : mt / 32;
+      for (int vt = 16; vt <= 128; vt += 16) {
+        if (mb * 3 * vt > 512 || (vt > cv && vt > 16)) break;
+        WgradPlan p{};
+        p.u_dy = u_dy;
+        p.mt = mt;
+        p.vt = vt;
+        p.mb = mb;
+        p.utiles = (cu + mt - 1) / mt;
+        p.vtiles = (cv + vt - 1) / vt;
+        const int k = (w + 127) / 128;
+        p.Wt = (w + k - 1) / k;
+        p.pitch = p.Wt + 2;
+        p.strips = (w + p.Wt - 1) / p.Wt;
+        p.len = ((long long)n * (h + 1) - 1) * p.pitch;
+        p.tmem = 32;
+        while (p.tmem < mb * 3 * vt) p.tmem *= 2;
+        for (int kp : {112, 48}) {   // KP + 2 positions of U fill whole passes of a producer group
+          p.KP = kp;
+          // plane lengths for 16-byte stores of a warp's positions and 16-channel groups without bank conflicts
+          // (two groups: 2 mod 4; more: odd)
+          auto pad = [](int len, int groups) {
+            const int want = groups <= 4 ? 2 : 1;   // groups of 8 channels
+            return len + ((want - len) % 8 + 8) % 8;
+          };
+          const int ucopies = mb == 3 ? 1 : 3;
+          p.ulen = pad(mb == 3 ? p.KP + 2 : p.KP, mt / 8);
+          p.u_bytes = (ucopies * mt / 8 * p.ulen * 16 + 127) / 128 * 128;
+          for (p.slots = kWgMaxSlots; p.slots >= 2; --p.slots) {
+            p.rv = p.slots * p.KP + 2 * p.pitch;
+            p.vlen = pad(p.rv + 16, vt / 8);
+            p.v_bytes = vt / 8 * p.vlen * 16;
+            // a product reads 16 planes of U from each block, also where fewer are staged: room for them behind
+            p.smem = kWgHead + p.slots * p.u_bytes + std::max(std::max(p.v_bytes, 16 * p.ulen * 16), 64 * kWgProd);
+            if (p.smem <= kCvSmem) break;
+          }
+          if (p.slots >= 3) break;
+        }
+        if (p.slots < 2) continue;
+        p.steps = (p.len + p.KP - 1) / p.KP;
+        const long long total = p.steps * p.strips, tiles = (long long)p.utiles * p.vtiles;
+        p.chunks = std::max(1LL, std::min(std::min(total, most), sms / tiles));
+        p.chunks = std::min<long long>(p.chunks, 9 * cin);         // room of the bias partials
+        const double waves = (double)((tiles * p.chunks + sms - 1) / sms);
+        const double load = 16.0 * 4 * (std::min(mt, cu) + std::min(vt, cv)) / 12.0;
+        const double mma = mb * 3 * (32.0 + vt / 4.0);
+        const double per = (double)total * p.KP / 16 / p.chunks;
+        const double cost = waves * (per * std::max(load, mma) + 2.0 * p.pitch / 16 * load) + 0.5 * p.chunks * 9;
+        if (best_cost < 0 || cost < best_cost) best = p, best_cost = cost;
+      }
+    }
+  }
+  WgradPlan& p = best;
+  const long long per = (p.steps * p.strips + p.chunks - 1) / p.chunks * p.KP;   // positions per chunk
+  const long long segs = std::max(1LL, (long long)((double)per / (1.1 * chain) + 0.999));
+  p.seg_steps = (int)std::min<long long>(((per + segs - 1) / segs + p.KP - 1) / p.KP, (1 << 22) / p.KP);
+  p.mp = (unsigned)(((1ull << 32) + p.pitch - 1) / p.pitch);
+  const long long rows = (long long)p.seg_steps * p.KP / p.pitch + 5;
+  p.mh = rows <= h ? 0u : (unsigned)(((1ull << 32) + h) / (h + 1));
+  p.bias_chunks = (pixels + kBiasChunk - 1) / kBiasChunk;
+  p.ws_chunks = p.chunks + 1;
+  return best;
 }
 
 }  // namespace
@@ -1174,7 +1284,7 @@ extern "C" {
 long long lbm_nn_wgrad_workspace(int n, int h, int w, int cin, int cout) {
   if (n < 1 || h < 1 || w < 1 || cin < 1 || cout < 1) return 0;
   const WgradPlan p = wgrad_plan(n, h, w, cin, cout);
-  return p.chunks * 9LL * cin * cout + p.bias_chunks * cout;
+  return p.ws_chunks * 9LL * cin * cout + p.bias_chunks * cout;
 }
 
 int lbm_nn_conv3x3_wgrad(const float* x, const float* dy, float* dw, float* db, float* work, long long work_len,
@@ -1185,46 +1295,25 @@ int lbm_nn_conv3x3_wgrad(const float* x, const float* dy, float* dw, float* db, 
   cudaStream_t s = (cudaStream_t)stream;
   const WgradPlan p = wgrad_plan(n, h, w, cin, cout);
   const long long nw = 9LL * cin * cout;
-  if (p.chunks > 65535) return -1;
-  static unsigned long long attr_set = 0;   // shared-memory opt-in, per device
+  static std::atomic<unsigned long long> attr_set{0};   // shared-memory opt-in, per device
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -3;
-  if (!(attr_set & (1ull << dev))) {
-    if (cudaFuncSetAttribute((const void*)conv3x3_wgrad_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             WgTcSmem<64>::bytes()) != cudaSuccess ||
-        cudaFuncSetAttribute((const void*)conv3x3_wgrad_tc<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             WgTcSmem<32>::bytes()) != cudaSuccess ||
-        cudaFuncSetAttribute((const void*)conv3x3_wgrad_tc_rows<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             WgRowsSmem<64>::bytes()) != cudaSuccess ||
-        cudaFuncSetAttribute((const void*)conv3x3_wgrad_tc_rows<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             WgRowsSmem<32>::bytes()) != cudaSuccess)
-      return -3;
-    attr_set |= 1ull << dev;
+  if (!(attr_set.load(std::memory_order_acquire) & (1ull << dev))) {
+    for (const void* fn : {(const void*)conv3x3_wgrad<1>, (const void*)conv3x3_wgrad<2>, (const void*)conv3x3_wgrad<3>})
+      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kCvSmem) != cudaSuccess) return -3;
+    attr_set.fetch_or(1ull << dev, std::memory_order_acq_rel);
   }
-  if (cout <= 64) {
-    const dim3 grid((cout + 31) / 32, (cin + kWtN - 1) / kWtN, (unsigned)p.chunks);
-    if (p.W == 64)
-      conv3x3_wgrad_tc_rows<64><<<grid, kWtThreads, WgRowsSmem<64>::bytes(), s>>>(x, dy, work, n, h, w, cin, cout,
-                                                                                  p.per_chunk);
-    else
-      conv3x3_wgrad_tc_rows<32><<<grid, kWtThreads, WgRowsSmem<32>::bytes(), s>>>(x, dy, work, n, h, w, cin, cout,
-                                                                                  p.per_chunk);
-  } else {
-    const dim3 grid((cout + kWtM - 1) / kWtM, 3 * ((cin + kWtN - 1) / kWtN), (unsigned)p.chunks);
-    if (p.W == 64)
-      conv3x3_wgrad_tc<64><<<grid, kWtThreads, WgTcSmem<64>::bytes(), s>>>(x, dy, work, n, h, w, cin, cout,
-                                                                           p.per_chunk);
-    else
-      conv3x3_wgrad_tc<32><<<grid, kWtThreads, WgTcSmem<32>::bytes(), s>>>(x, dy, work, n, h, w, cin, cout,
-                                                                           p.per_chunk);
-  }
-  sum_parts<<<(unsigned)((nw + 31) / 32), 256, 0, s>>>(work, dw, nw, (int)p.chunks);
-  if (db) {
-    float* bpart = work + p.chunks * nw;
-    const long long P = (long long)n * h * w;
-    colsum_part<<<dim3((cout + 31) / 32, (unsigned)p.bias_chunks), 256, 0, s>>>(dy, bpart, P, cout, kBiasChunk);
-    sum_parts<<<(unsigned)((cout + 31) / 32), 256, 0, s>>>(bpart, db, cout, (int)p.bias_chunks);
-  }
+  float* bpart = work + p.chunks * nw;
+  const WgradArgs a{p.u_dy ? dy : x, p.u_dy ? x : dy, work, db ? bpart : nullptr, n, h, w,
+                    p.u_dy ? cout : cin, p.u_dy ? cin : cout, cin, cout,
+                    ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 31) == 0, p};
+  const unsigned grid = (unsigned)(p.chunks * p.utiles * p.vtiles);
+  if (p.mb == 1) conv3x3_wgrad<1><<<grid, kWgThreads, p.smem, s>>>(a);
+  else if (p.mb == 2) conv3x3_wgrad<2><<<grid, kWgThreads, p.smem, s>>>(a);
+  else conv3x3_wgrad<3><<<grid, kWgThreads, p.smem, s>>>(a);
+  const int nb = db ? cout : 0;
+  const int lanes = p.chunks > 64 ? kSumLanes : (p.chunks > 32 ? 8 : (p.chunks > 12 ? 4 : 2));
+  sum_parts<<<(unsigned)((nw + 31) / 32 + (nb + 31) / 32), 32 * lanes, 0, s>>>(work, dw, nw, bpart, db, nb, (int)p.chunks);
   return status(cudaGetLastError());
 }
 
