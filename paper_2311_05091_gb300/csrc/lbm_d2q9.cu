@@ -169,32 +169,22 @@ __device__ __forceinline__ Nat natural_of(const Her& h, float cs2, float cs4) {
 // history = (phi1, 0, 0, 0, 0)
 // ---------------------------------------------------------------------------
 template <typename GT>
-__global__ void d2q9_init(const float* __restrict__ phi0_all, const float* __restrict__ phi1_all,
-                          float* __restrict__ f_all, GT* __restrict__ g_all, float* __restrict__ hist_all,
-                          const InstanceConsts* __restrict__ consts, int nx, int ny, int per_x, int per_y) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y;
-  const int b = blockIdx.z;
-  if (x >= nx) return;
-  const InstanceConsts& k = consts[b];
+__device__ __forceinline__ void init_node(const InstanceConsts& k, const float* __restrict__ phi0,
+                                          const float* __restrict__ phi1, float* __restrict__ f, GT* __restrict__ g,
+                                          float* __restrict__ h, int x, int y, int nx, int ny, int per_x, int per_y) {
   const long long plane = (long long)nx * ny;
-  const float* phi0 = phi0_all + (long long)b * plane;
-  const float* phi1 = phi1_all + (long long)b * 5 * plane;   // staged in a history plane
-  auto at = [&](const float* a, int dx, int dy) {
-    const int xx = wrap_or_mirror(x + dx, nx, per_x), yy = wrap_or_mirror(y + dy, ny, per_y);
-    return a[(long long)yy * nx + xx];
+  // the neighbours' rows and columns, without a division
+  const int xm = wrap_or_mirror_row(x - 1, nx, per_x), xp = wrap_or_mirror_row(x + 1, nx, per_x);
+  const long long rm = (long long)wrap_or_mirror_row(y - 1, ny, per_y) * nx, r0 = (long long)y * nx,
+                  rp = (long long)wrap_or_mirror_row(y + 1, ny, per_y) * nx;
+  auto hood = [&](const float* a) {
+    return P9{a[r0 + x], a[r0 + xp], a[rp + x], a[r0 + xm], a[rm + x], a[rp + xp], a[rp + xm], a[rm + xm], a[rm + xp]};
   };
-  P9 v0{at(phi0, 0, 0), at(phi0, 1, 0), at(phi0, 0, 1), at(phi0, -1, 0), at(phi0, 0, -1),
-        at(phi0, 1, 1), at(phi0, -1, 1), at(phi0, -1, -1), at(phi0, 1, -1)};
-  P9 v1{at(phi1, 0, 0), at(phi1, 1, 0), at(phi1, 0, 1), at(phi1, -1, 0), at(phi1, 0, -1),
-        at(phi1, 1, 1), at(phi1, -1, 1), at(phi1, -1, -1), at(phi1, 1, -1)};
+  const P9 v0 = hood(phi0), v1 = hood(phi1);
   float mu0, mu1, mu2;
   chem_pot(k, v0.c, v1.c, iso_lap(v0), iso_lap(v1), mu0, mu1, mu2);
   const float emb = k.eta * mubar1_of(k, mu0, mu1, mu2);
-  const long long node = (long long)y * nx + x;
-  float* f = f_all + (long long)b * 9 * plane;
-  GT* g = g_all + (long long)b * 9 * plane;
-  float* h = hist_all + (long long)b * 5 * plane;
+  const long long node = r0 + x;
   f[node] = v1.c + (k.w0 - 1.f) * emb;
 #pragma unroll
   for (int i = 1; i < 9; ++i) f[(long long)i * plane + node] = (i < 5 ? k.wa : k.we) * emb;
@@ -203,6 +193,51 @@ __global__ void d2q9_init(const float* __restrict__ phi0_all, const float* __res
   h[node] = v1.c;
 #pragma unroll
   for (int q = 1; q < 5; ++q) h[(long long)q * plane + node] = 0.f;
+}
+
+template <typename GT>
+__global__ void d2q9_init(const float* __restrict__ phi0_all, const float* __restrict__ phi1_all,
+                          float* __restrict__ f_all, GT* __restrict__ g_all, float* __restrict__ hist_all,
+                          const InstanceConsts* __restrict__ consts, int nx, int ny, int per_x, int per_y) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int b = blockIdx.z;
+  if (x >= nx) return;
+  const long long plane = (long long)nx * ny;
+  init_node(consts[b], phi0_all + (long long)b * plane, phi1_all + (long long)b * 5 * plane,   // staged in a history plane
+            f_all + (long long)b * 9 * plane, g_all + (long long)b * 9 * plane, hist_all + (long long)b * 5 * plane, x,
+            (int)blockIdx.y, nx, ny, per_x, per_y);
+}
+
+// The instances of a multi-size context in one launch, a CTA per work item of the step (args: launch arguments of the
+// step that will start from the buffers initialised here).  phi1: the instances' fields back to back, as phi0 from
+// phi0_base on.  64 uneven lattices took a copy and a launch each.
+template <typename GT>
+__global__ void d2q9_init_items(const StepArgs* __restrict__ args, const int4* __restrict__ items,
+                                const float* __restrict__ phi0_base, const float* __restrict__ phi1) {
+  const int4 w = items[blockIdx.x];
+  const StepArgs a = args[w.x];
+  const int x = w.y + threadIdx.x;
+  if (x >= a.nx) return;
+  for (int y = w.z; y < min(w.z + a.strip, a.ny); ++y)
+    init_node(*a.consts, a.phi0, phi1 + (a.phi0 - phi0_base), const_cast<float*>(a.f_in),
+              static_cast<GT*>(const_cast<void*>(a.g_in)), const_cast<float*>(a.hist_in), x, y, a.nx, a.ny, a.per_x,
+              a.per_y);
+}
+
+// phi1 and u of every instance of a multi-size context, back to back: [offset] and [2 offset], offsets as phi0's
+__global__ void d2q9_pack_items(const StepArgs* __restrict__ args, const int4* __restrict__ items,
+                                const float* __restrict__ phi0_base, float* __restrict__ phi1, float* __restrict__ u) {
+  const int4 w = items[blockIdx.x];
+  const StepArgs a = args[w.x];
+  const int x = w.y + threadIdx.x;
+  if (x >= a.nx) return;
+  const long long o = a.phi0 - phi0_base, n = a.nodes;
+  for (int y = w.z; y < min(w.z + a.strip, a.ny); ++y) {
+    const long long node = (long long)y * a.nx + x;
+    phi1[o + node] = a.hist_in[node];
+    u[2 * o + node] = a.hist_in[n + node];
+    u[2 * o + n + node] = a.hist_in[2 * n + node];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -741,6 +776,19 @@ cudaError_t launch_d2q9_init(const float* phi0, const float* phi1, float* f, voi
   else
     d2q9_init<float><<<grid, block, 0, s>>>(phi0, phi1, f, static_cast<float*>(g), hist, consts, nx, ny, per_x,
                                             per_y);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_d2q9_init_items(const StepArgs* args, const int4* items, int nitems, const float* phi0,
+                                   const float* phi1, int g_half, cudaStream_t s) {
+  if (g_half) d2q9_init_items<__half><<<nitems, BX, 0, s>>>(args, items, phi0, phi1);
+  else d2q9_init_items<float><<<nitems, BX, 0, s>>>(args, items, phi0, phi1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_d2q9_pack_items(const StepArgs* args, const int4* items, int nitems, const float* phi0, float* phi1,
+                                   float* u, cudaStream_t s) {
+  d2q9_pack_items<<<nitems, BX, 0, s>>>(args, items, phi0, phi1, u);
   return cudaGetLastError();
 }
 

@@ -94,6 +94,12 @@ cudaError_t launch_d2q9_init(const float* phi0, const float* phi1, float* f, voi
                              float* hist, const InstanceConsts* consts, int nx, int ny,
                              int per_x, int per_y, int nbatch, cudaStream_t s);
 cudaError_t launch_d2q9_step(const StepArgs& a, int nbatch, bool observe, cudaStream_t s);
+// Multi-size contexts: initial state of every instance from the fields phi1 (back to back, like phi0), and their
+// phi1 and u gathered back to back; args and items as for launch_d2q9_items.
+cudaError_t launch_d2q9_init_items(const StepArgs* args, const int4* items, int nitems, const float* phi0,
+                                   const float* phi1, int g_half, cudaStream_t s);
+cudaError_t launch_d2q9_pack_items(const StepArgs* args, const int4* items, int nitems, const float* phi0, float* phi1,
+                                   float* u, cudaStream_t s);
 // Work-list form for instances of different sizes: args[inst] holds the
 // instance's own base pointers, sizes and strip (device memory), items[k] =
 // (inst, x0, ys, 0).  grid <= 0 picks a persistent grid of SMs x occupancy.
@@ -129,15 +135,17 @@ int build_d3q19_maps(const void* g, int g_half, const float* mom, const float* h
 
 // Observables: deterministic two-pass reduction of one instance.
 //   phi0, phi1, u (d planes), p: device fields of one instance, n nodes.
-//   partials: scratch of obs_partials_len(n) doubles.  out: 8 doubles
-//   [sum phi1, sum phi0, max|u|, sum p_in, n_in, sum p_out, n_out, nonfinite].
+//   partials: scratch of obs_partials_len(n) doubles.  out: kObsRecord doubles
+//   [sum phi1, sum phi0, max|u|, sum p_in, n_in, sum p_out, n_out, nonfinite,
+//   status flag], then 2 ncol floats: every stride-th value of col1 and of col0.
+constexpr int kObsRecord = 10;   // doubles (even, so the floats behind stay aligned)
 int obs_partials_blocks(long long n);
 long long obs_partials_len(long long n);
-// Pore-space phase fluxes of one instance along one axis (ua: that velocity component), 8 doubles to out.
+// Pore-space phase fluxes of one instance along one axis (ua: that velocity component), kObsRecord doubles to out.
 cudaError_t launch_phase_flux(const float* phi0, const float* phi1, const float* ua, long long n, double* partials,
-                              double* out, cudaStream_t s);
+                              double* out, const unsigned int* flag, cudaStream_t s);
 cudaError_t launch_observables(const float* phi0, const float* phi1, const float* u, int d,
-                               const float* p, long long n, double* partials, double* out,
-                               cudaStream_t s);
+                               const float* p, long long n, double* partials, double* out, const unsigned int* flag,
+                               const float* col1, const float* col0, int stride, int ncol, cudaStream_t s);
 
 }  // namespace lbm

@@ -84,8 +84,16 @@ __global__ void __launch_bounds__(kThreads) obs_pass1(const float* __restrict__ 
   }
 }
 
+// Second pass: the records of pass 1, the context's status flag behind them (out[8]), and, when `ncol` > 0, the
+// columns a contact angle is read from (every `stride`-th value of col1, then of col0) behind that, so that the host
+// needs one copy and one wait for all of it.
 __global__ void __launch_bounds__(kThreads) obs_pass2(const double* __restrict__ partials, int nblocks,
-                                                      double* __restrict__ out) {
+                                                      double* __restrict__ out, const unsigned int* __restrict__ flag,
+                                                      const float* __restrict__ col1, const float* __restrict__ col0,
+                                                      int stride, int ncol) {
+  float* cols = reinterpret_cast<float*>(out + kObsRecord);
+  for (int k = threadIdx.x; k < 2 * ncol; k += blockDim.x)
+    cols[k] = k < ncol ? col1[(long long)k * stride] : col0[(long long)(k - ncol) * stride];
   __shared__ double sh[kThreads / 32][kRec];
   double v[kRec] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
@@ -99,6 +107,7 @@ __global__ void __launch_bounds__(kThreads) obs_pass2(const double* __restrict__
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int q = 0; q < kRec; ++q) out[q] = v[q];
+    out[kRec] = (double)*flag;
   }
 }
 
@@ -138,12 +147,12 @@ __global__ void __launch_bounds__(kThreads) flux_pass1(const float* __restrict__
 }  // namespace
 
 cudaError_t launch_phase_flux(const float* phi0, const float* phi1, const float* ua, long long n, double* partials,
-                              double* out, cudaStream_t s) {
+                              double* out, const unsigned int* flag, cudaStream_t s) {
   const int nb = obs_partials_blocks(n);
   flux_pass1<<<nb, kThreads, 0, s>>>(phi0, phi1, ua, n, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  obs_pass2<<<1, kThreads, 0, s>>>(partials, nb, out);
+  obs_pass2<<<1, kThreads, 0, s>>>(partials, nb, out, flag, nullptr, nullptr, 0, 0);
   return cudaGetLastError();
 }
 
@@ -157,12 +166,13 @@ int obs_partials_blocks(long long n) {
 long long obs_partials_len(long long n) { return (long long)obs_partials_blocks(n) * kRec; }
 
 cudaError_t launch_observables(const float* phi0, const float* phi1, const float* u, int d, const float* p,
-                               long long n, double* partials, double* out, cudaStream_t s) {
+                               long long n, double* partials, double* out, const unsigned int* flag, const float* col1,
+                               const float* col0, int stride, int ncol, cudaStream_t s) {
   const int nb = obs_partials_blocks(n);
   obs_pass1<<<nb, kThreads, 0, s>>>(phi0, phi1, u, d, p, n, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  obs_pass2<<<1, kThreads, 0, s>>>(partials, nb, out);
+  obs_pass2<<<1, kThreads, 0, s>>>(partials, nb, out, flag, col1, col0, stride, ncol);
   return cudaGetLastError();
 }
 
