@@ -219,7 +219,8 @@ int lbm_create_multi(lbm_lattice lattice, int ninst, const int* nx, const int* n
 /* Shape and node offset of one instance (any context). */
 int lbm_get_instance_shape(const lbm_ctx* ctx, int instance, int* nx, int* ny, int64_t* offset);
 
-/* Launch autotuner: chooses the row strip (of every size class of a
+/* Launch autotuner: chooses the row strip (or keeps the tiles of a small
+ * lattice, where they are faster than every strip; of every size class of a
  * multi-size context, or the context's single strip) among 4, 8, 12, 16, 18,
  * 20, 24, 32, 48, 64 by timing `trial` steps per candidate, two
  * coordinate-descent passes.  The
@@ -239,7 +240,10 @@ int lbm_set_stream(lbm_ctx* ctx, void* stream);
 /* Launch tuning; results do not depend on it (bitwise).  strip >= 1: rows
  * (D2Q9) or z planes (D3Q19) swept by one CTA of the step kernel; by default
  * 16 rows or 32 planes, or, when that gives fewer CTAs than two waves on the
- * device, the shorter strip a wave model picks.  depth in
+ * device, the shorter strip a wave model picks; a D2Q9 context of one size
+ * that was given no strip and has at most 2.5 million nodes (or rows that are
+ * not a multiple of four nodes) runs tiles of one node per thread instead of
+ * swept strips.  depth in
  * 1..3 (0 keeps the current value): D2Q9, rows of asynchronous
  * global-to-shared copies each CTA keeps in flight (default 1); D3Q19, 1
  * selects the generic fused kernel (synchronous halo loads), 2 or 3 the

@@ -50,6 +50,7 @@ struct lbm_ctx {
   int per[3] = {0, 0, 0};
   long long nodes = 0;        // per instance
   int strip = 32;
+  int tile = 0;               // D2Q9: tile rows of the small-lattice kernel, 0: the sweep (always once a strip is set)
   int depth = 1;
   int wait_polls = lbm::kWaitPollsDefault;   // lbm_set_wait_limit
   int device = 0;             // CUDA device the context was created on
@@ -324,6 +325,20 @@ int default_strip(const lbm_ctx* c) {
   return (int)std::max(1LL, strip);
 }
 
+// Tile rows of the small-lattice D2Q9 kernel where it is the faster form, else 0: up to 2.5 M nodes (1024^2 x 2: 94 us
+// against 99 of the sweep at its default strip, x 3: 140 against 145, or 131 tuned), and at every size where the rows
+// are not on 16 bytes and the sweep has to copy them word by word (1023^2 x 2: 97 against 106).  Four rows while those
+// CTAs stay below four per SM, else eight.
+int default_tile(const lbm_ctx* c) {
+  if (c->lattice != LBM_D2Q9 || c->multi) return 0;
+  if (c->total > 2500000 && c->nx % 4 == 0) return 0;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) return 0;
+  const long long ctas = (long long)((c->nx + 31) / 32) * ((c->ny + 3) / 4) * c->nbatch;
+  // grids are limited to 65535 rows of tiles
+  return ctas < 4LL * sms ? 4 : (c->ny <= 8 * 65535 ? 8 : 0);
+}
+
 StepArgs step_args(lbm_ctx* c, int from) {
   StepArgs a;
   a.f_in = c->f[from];
@@ -344,6 +359,7 @@ StepArgs step_args(lbm_ctx* c, int from) {
   a.per_y = c->per[1];
   a.per_z = c->per[2];
   a.strip = c->strip;
+  a.tile = c->tile;
   a.depth = c->depth;
   a.wait_polls = c->wait_polls;
   a.s_zero = 1;
@@ -742,6 +758,7 @@ static int create_impl(lbm_lattice lattice, int nbatch, const int* nxs, const in
     return cuda_fail(nullptr, e, "cudaGetDevice");
   }
   c->strip = default_strip(c);
+  c->tile = default_tile(c);
   c->depth = is3d ? 2 : 1;
   c->g_half = g_half;
   c->g_elem = g_half ? sizeof(__half) : sizeof(float);
@@ -880,6 +897,7 @@ int lbm_set_launch(lbm_ctx* c, int strip, int depth) {
   if (depth < 0 || depth > 3) return set_err(c, LBM_EINVAL, "depth must lie in 0..3 (0 keeps the current)");
   LBM_CK(c, cudaStreamSynchronize(c->stream));
   c->strip = strip;
+  c->tile = 0;
   if (depth > 0) c->depth = depth;
   drop_graphs(c);
   if (c->multi) {
@@ -934,6 +952,7 @@ int lbm_tune(lbm_ctx* c, int trial, int* strips_out) {
       }
     if (!placed) classes.push_back({b});
   }
+  const int tile0 = c->tile;          // the small-lattice kernel, when the context uses it, against every strip
   auto apply = [&](int cl, int strip) -> cudaError_t {
     if (c->multi) {
       for (int b : classes[cl]) c->istrip[b] = std::min(strip, c->iny[b]);
@@ -960,6 +979,9 @@ int lbm_tune(lbm_ctx* c, int trial, int* strips_out) {
   // (its CTA count is three full waves of 152 SMs x 5 CTAs), 1.8 % faster than 16
   static const int cand[] = {4, 8, 12, 16, 18, 20, 24, 32, 48, 64};
   constexpr int ncand = (int)(sizeof(cand) / sizeof(cand[0]));
+  float tile_ms = 1e30f, sweep_ms = 1e30f;
+  if (tile0) e = measure(tile_ms);
+  c->tile = 0;
   for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
     for (int cl = 0; cl < (int)classes.size() && e == cudaSuccess; ++cl) {
       const int rows = c->multi ? c->iny[classes[cl][0]] : (c->lattice == LBM_D2Q9 ? c->ny : c->nz);
@@ -977,9 +999,11 @@ int lbm_tune(lbm_ctx* c, int trial, int* strips_out) {
         }
       }
       if (e == cudaSuccess) e = apply(cl, best);
+      sweep_ms = std::min(sweep_ms, best_ms);
       if (!c->multi) break;   // one strip for the whole context
     }
   }
+  if (tile0 && tile_ms < sweep_ms) c->tile = tile0;
   // restore the state the tuner found
   c->cur = cur0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(c->f[cur0], sf, pop, cudaMemcpyDeviceToDevice, c->stream);

@@ -35,19 +35,18 @@ namespace {
 //        11 (+x,+z), 12 (-x,-z), 13 (+x,-z), 14 (-x,+z), 15 (+y,+z), 16 (-y,-z), 17 (+y,-z), 18 (-y,+z).
 // D3Q15: 0, 1-6 axes as D3Q19, 7-14 corners (1,1,1) (-1,1,1) (1,-1,1) (-1,-1,1) (1,1,-1) (-1,1,-1)
 //        (1,-1,-1) (-1,-1,-1).
-__constant__ signed char kC9[9][3] = {{0, 0, 0}, {1, 0, 0},  {0, 1, 0},  {-1, 0, 0}, {0, -1, 0},
+template <int Q>
+__device__ __forceinline__ constexpr int cvel(int i, int a) {
+  constexpr signed char c9[9][3] = {{0, 0, 0}, {1, 0, 0},  {0, 1, 0},  {-1, 0, 0}, {0, -1, 0},
                                       {1, 1, 0}, {-1, 1, 0}, {-1, -1, 0}, {1, -1, 0}};
-__constant__ signed char kC19[19][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
+  constexpr signed char c19[19][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
                                         {0, 0, 1},  {0, 0, -1}, {1, 1, 0},  {-1, -1, 0}, {1, -1, 0},
                                         {-1, 1, 0}, {1, 0, 1},  {-1, 0, -1}, {1, 0, -1}, {-1, 0, 1},
                                         {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
-__constant__ signed char kC15[15][3] = {{0, 0, 0}, {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0},
+  constexpr signed char c15[15][3] = {{0, 0, 0}, {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0},
                                         {0, 0, 1}, {0, 0, -1}, {1, 1, 1},  {-1, 1, 1}, {1, -1, 1},
                                         {-1, -1, 1}, {1, 1, -1}, {-1, 1, -1}, {1, -1, -1}, {-1, -1, -1}};
-
-template <int Q>
-__device__ __forceinline__ int cvel(int i, int a) {
-  return Q == 9 ? kC9[i][a] : (Q == 19 ? kC19[i][a] : kC15[i][a]);
+  return Q == 9 ? c9[i][a] : (Q == 19 ? c19[i][a] : c15[i][a]);
 }
 
 template <class GT>
@@ -61,7 +60,9 @@ __device__ __forceinline__ void gstore(GT* p, float v, const InstanceConsts& k) 
   else *p = v;
 }
 
-// One thread per boundary node: blockIdx.y = side (0 inlet, 1 outlet), blockIdx.z = instance.
+// One thread per boundary node: blockIdx.y = side (0 inlet, 1 outlet), blockIdx.z = instance.  A few thousand nodes at
+// most: latency is all there is, so the velocities are compile-time constants, a warp is a CTA, and with programmatic
+// launch the CTAs wait for the step where they stand.
 template <int Q, class GT>
 __global__ void inout_kernel(float* __restrict__ f, GT* __restrict__ g, const float* __restrict__ phi0,
                              const InstanceConsts* __restrict__ consts, const float* __restrict__ u_in, int mode,
@@ -70,8 +71,10 @@ __global__ void inout_kernel(float* __restrict__ f, GT* __restrict__ g, const fl
   const long long cols = (long long)ny * nz;
   const long long col = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int side = blockIdx.y, b = blockIdx.z;
-  if (col >= cols || !(mode & (1 << side))) return;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const InstanceConsts k = consts[b];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (col >= cols || !(mode & (1 << side))) return;
   const int xb = side == 0 ? 0 : nx - 1, xf = side == 0 ? 1 : nx - 2;
   const long long nb = col * nx + xb, nf = col * nx + xf;
   float* fb = f + (long long)b * Q * nodes;
@@ -141,14 +144,20 @@ cudaError_t launch_q(float* f, void* g, int g_half, const float* phi0, const Ins
                      const float* u_in, int mode, float phi_in, float p_out, int nx, int ny, int nz, long long nodes,
                      int nbatch, cudaStream_t s) {
   const long long cols = (long long)ny * nz;
-  dim3 grid((unsigned)((cols + 127) / 128), 2, nbatch);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((cols + 31) / 32), 2, nbatch);
+  cfg.blockDim = dim3(32);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   if (g_half)
-    inout_kernel<Q, __half><<<grid, 128, 0, s>>>(f, static_cast<__half*>(g), phi0, consts, u_in, mode, phi_in,
-                                                 p_out, nx, ny, nz, nodes);
-  else
-    inout_kernel<Q, float><<<grid, 128, 0, s>>>(f, static_cast<float*>(g), phi0, consts, u_in, mode, phi_in, p_out,
-                                                nx, ny, nz, nodes);
-  return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, inout_kernel<Q, __half>, f, static_cast<__half*>(g), phi0, consts, u_in, mode, phi_in,
+                              p_out, nx, ny, nz, nodes);
+  return cudaLaunchKernelEx(&cfg, inout_kernel<Q, float>, f, static_cast<float*>(g), phi0, consts, u_in, mode, phi_in,
+                            p_out, nx, ny, nz, nodes);
 }
 
 }  // namespace

@@ -95,6 +95,49 @@ __device__ __forceinline__ float mubar1_of(const InstanceConsts& k, float mu0, f
   return k.gT3 * ((mu1 - mu0) * k.inv_gam0 + (mu1 - mu2) * k.inv_gam2);
 }
 
+// Chemical potentials of one point: mubar_1 and the differences mu0 - mu2, mu1 - mu2 the forces use.  Every rounding is
+// spelled out, so that the kernel forms of the step agree bitwise and a change of one does not re-round the others.
+// EDGE: the point lies in the halo column of a 128-column tile of the sweep, where the compiler contracted the two
+// differences of mubar_1 the other way; kept, so that results stay what they were (a run with FP16 populations turns
+// one such rounding into another history).
+__device__ __forceinline__ float lap_rn(const P9& v) {
+  const float a = (v.e - v.c) + (v.w - v.c) + (v.n - v.c) + (v.s - v.c);
+  const float d = (v.ne - v.c) + (v.nw - v.c) + (v.sw - v.c) + (v.se - v.c);
+  return __fmaf_rn(a, 2.f / 3.f, __fmul_rn(d, 1.f / 6.f));
+}
+template <bool EDGE>
+__device__ __forceinline__ void mu_point(const InstanceConsts& k, const P9& v0, const P9& v1, float& mub, float& d02,
+                                         float& d12) {
+  const float ph0 = v0.c, ph1 = v1.c, ph2 = __fsub_rn(__fsub_rn(1.f, ph0), ph1);
+  const float lap0 = lap_rn(v0), lap1 = lap_rn(v1), lap2 = __fsub_rn(-lap0, lap1);
+  auto psi = [&](float ph, float lap) {
+    const float x = __fmul_rn(__fmul_rn(k.c12_W, ph), __fsub_rn(1.f, ph)), y = __fmaf_rn(-2.f, ph, 1.f);
+    return __fmaf_rn(x, y, -__fmul_rn(k.c34_W, lap));
+  };
+  const float psi0 = psi(ph0, lap0), psi1 = psi(ph1, lap1), psi2 = psi(ph2, lap2);
+  const float mu0 = __fmul_rn(k.gam0, psi0), mu1 = __fmul_rn(k.gam1, psi1), mu2 = __fmul_rn(k.gam2, psi2);
+  d02 = __fsub_rn(mu0, mu2);
+  d12 = EDGE ? __fmaf_rn(-k.gam2, psi2, mu1) : __fmaf_rn(k.gam1, psi1, -mu2);
+  const float d10 = EDGE ? __fmaf_rn(-k.gam0, psi0, mu1) : __fmaf_rn(k.gam1, psi1, -mu0);
+  mub = __fmul_rn(k.gT3, __fmaf_rn(d10, k.inv_gam0, __fmul_rn(d12, k.inv_gam2)));
+}
+// S_x u_y - u_x S_y of the previous step, the correction force's product
+__device__ __forceinline__ float correction_product(float sx, float uy, float ux, float sy) {
+  return __fmaf_rn(sx, uy, -__fmul_rn(ux, sy));
+}
+
+// phi1 = sum f and the first moment j of nine CH populations.
+__device__ __forceinline__ float phase_sum(const float (&v)[9]) {
+  float sum = v[0];
+#pragma unroll
+  for (int i = 1; i < 9; ++i) sum += v[i];
+  return sum;
+}
+__device__ __forceinline__ void first_moment(const float (&v)[9], float& jx, float& jy) {
+  jx = (v[1] - v[3]) + (v[5] - v[6]) - (v[7] - v[8]);
+  jy = (v[2] - v[4]) + (v[5] + v[6]) - (v[7] + v[8]);
+}
+
 // Natural moments (rows of M0, Appendix A) of nine populations.
 struct Nat {
   float m0, mx, my, mxx, myy, mxy, mxyy, mxxy, mxxyy;
@@ -185,9 +228,10 @@ __device__ __forceinline__ void init_node(const InstanceConsts& k, const float* 
   chem_pot(k, v0.c, v1.c, iso_lap(v0), iso_lap(v1), mu0, mu1, mu2);
   const float emb = k.eta * mubar1_of(k, mu0, mu1, mu2);
   const long long node = r0 + x;
+  const float fa = k.wa * emb, fe = k.we * emb;   // before the stores, which could alias the constants
   f[node] = v1.c + (k.w0 - 1.f) * emb;
 #pragma unroll
-  for (int i = 1; i < 9; ++i) f[(long long)i * plane + node] = (i < 5 ? k.wa : k.we) * emb;
+  for (int i = 1; i < 9; ++i) f[(long long)i * plane + node] = i < 5 ? fa : fe;
 #pragma unroll
   for (int i = 0; i < 9; ++i) g[(long long)i * plane + node] = GT(0.f);
   h[node] = v1.c;
@@ -306,6 +350,192 @@ struct StepSmem {
 
 template <int D, typename GT>
 constexpr size_t step_smem_bytes() { return sizeof(StepSmem<D, GT>); }
+
+// Node update: gradients, forces, velocity, pressure, both collisions and the push stores, from the neighbourhoods of
+// phi1, phi0, mubar_1 and the correction-force product, the chemical-potential differences of the node, the first
+// moment j of its CH populations, its NS populations and its previous step.  Every kernel form of the step calls it
+// with the same values, so that they agree bitwise.
+template <bool OBS, typename GT, bool PER>
+__device__ __forceinline__ void collide_node(const StepArgs& a, const InstanceConsts& k, const int b, const int node,
+                                             const int x, const int y, const P9& v1, const P9& v0, const P9& vm,
+                                             const P9& va, const float d02, const float d12, const float jx,
+                                             const float jy, const float (&g)[9], const float php, const float uxp,
+                                             const float uyp, const float Sxp, const float Syp,
+                                             const float* __restrict__ f_in, float* __restrict__ f_out,
+                                             GT* __restrict__ g_out, float* __restrict__ h_out) {
+  const int nx = a.nx, ny = a.ny, per_x = a.per_x, per_y = a.per_y;
+  const long long plane = a.nodes;
+  const int pl = (int)plane;
+  const float cs2 = k.cs2, cs4 = k.cs4;
+  const float ph1 = v1.c, ph0 = v0.c, ph2 = 1.f - ph0 - ph1;
+  float g1x, g1y, g0x, g0y, gmx, gmy, dAx, dAy;
+  iso_grad(v1, g1x, g1y);
+  iso_grad(v0, g0x, g0y);
+  iso_grad(vm, gmx, gmy);
+  iso_grad(va, dAx, dAy);
+  const float mub = vm.c;
+
+  // degenerate mobility, mass flux S (frozen phi0), mixture properties
+  const float fdeg = ph1 * (1.f - ph1) * (1.f - ph0);
+  const float mob = k.M_cst + k.M_deg * fdeg;
+  const float sfac = (k.rho1 - k.rho2) * mob * k.inv_gam1;
+  const float Sx = sfac * gmx, Sy = sfac * gmy;
+  const float rho = k.rho0 * ph0 + k.rho1 * ph1 + k.rho2 * ph2;
+  const float grx = (k.rho0 - k.rho2) * g0x + (k.rho1 - k.rho2) * g1x;
+  const float gry = (k.rho0 - k.rho2) * g0y + (k.rho1 - k.rho2) * g1y;
+  const float muv = k.mu0 * ph0 + k.mu1 * ph1 + k.mu2 * ph2;
+
+  // F = F_s + F_b + F_c, F_s = (mu0 - mu2) grad phi0 + (mu1 - mu2) grad phi1
+  const float one_m0 = 1.f - ph0;
+  const float Fx = d02 * g0x + d12 * g1x + one_m0 * k.bx - 0.5f * dAy;
+  const float Fy = d02 * g0y + d12 * g1y + one_m0 * k.by + 0.5f * dAx;
+
+  // NS moments, velocity with the solid penalisation force
+  const Nat ng = natural(g);
+  const float inv_rho = __frcp_rn(rho);
+  const float usx = (ng.mx + 0.5f * Fx) * inv_rho;
+  const float usy = (ng.my + 0.5f * Fy) * inv_rho;
+  const float damp = 1.f - 0.5f * ph0;
+  const float ux = usx * damp, uy = usy * damp;
+  const float Ftx = Fx - ph0 * rho * usx, Fty = Fy - ph0 * rho * usy;
+
+  // local viscous rates (s0 = s4 = s2a)
+  const float om = fmaxf(one_m0, kOneMinusPhi0Floor);
+  // 1/s2a = 1/2 + mu / (rho (1 - phi0) a2a), likewise s2b; IEEE-rounded reciprocals
+  const float nu_e = muv * __frcp_rn(rho * om);
+  const float inv_s2a = 0.5f + nu_e * k.ia2a;
+  const float s2a = __frcp_rn(inv_s2a);
+  const float s2b = __frcp_rn(0.5f + nu_e * k.ia2b);
+
+  // pressure
+  const float udg = ux * grx + uy * gry;
+  const float q = (rho * ux - Sx) * ux + (rho * uy - Sy) * uy;
+  const float rhop = k.rho0 * ph0 + k.rho1 * php + k.rho2 * (1.f - ph0 - php);
+  const float qp = (rhop * uxp - Sxp) * uxp + (rhop * uyp - Syp) * uyp;
+  const float H = k.Kp * ((k.h0 - k.h2) * inv_s2a + k.h3);
+  const float sum_nz = ng.m0 - g[0];
+  const float p = k.pf * (sum_nz + (0.5f + H) * udg - k.wq * q + 0.5f * k.Kp * (q - qp));
+
+  // destinations of the nine pushes without branches: per axis and sign the
+  // neighbour's offset (periodic wrap folded in) and whether a wall reflects
+  const bool wxp = !PER && x + 1 >= nx && !per_x, wxm = !PER && x == 0 && !per_x;
+  const bool wyp = !PER && y + 1 >= ny && !per_y, wym = !PER && y == 0 && !per_y;
+  const int oxp = x + 1 < nx ? 1 : 1 - nx, oxm = x > 0 ? -1 : nx - 1;
+  const int oyp = y + 1 < ny ? nx : nx - pl, oym = y > 0 ? -nx : pl - nx;
+  auto store = [&](auto* __restrict__ out, int i, int io, int cx, int cy, float v) {
+    int off = 0;
+    bool bb = false;
+    if (cx) { off += cx > 0 ? oxp : oxm; bb = bb || (cx > 0 ? wxp : wxm); }
+    if (cy) { off += cy > 0 ? oyp : oym; bb = bb || (cy > 0 ? wyp : wym); }
+    g_store(out + (bb ? io * pl + node : i * pl + node + off), v, k);
+  };
+
+  // ---- NS collision in Hermite space ----
+  {
+    const Her h = hermite(ng, cs2, cs4);
+    const float exx = p + rho * ux * ux - Sx * ux;
+    const float eyy = p + rho * uy * uy - Sy * uy;
+    const float exy = rho * ux * uy - 0.5f * (Sx * uy + ux * Sy);
+    const float e4 = -cs2 * p;
+    const float dSxx = Sx * ux - Sxp * uxp;
+    const float dSyy = Sy * uy - Syp * uyp;
+    const float dSxy = 0.5f * (Sx * uy + ux * Sy) - 0.5f * (Sxp * uyp + uxp * Syp);
+    const float iso = (1.f - 3.f * cs2) * udg;
+    const float Mxx = 2.f * ux * Fx - dSxx + 2.f * cs2 * ux * grx + iso;
+    const float Myy = 2.f * uy * Fy - dSyy + 2.f * cs2 * uy * gry + iso;
+    const float Mxy = ux * Fy + Fx * uy - dSxy + cs2 * (ux * gry + grx * uy);
+    Her o;
+    o.h0 = h.h0 - s2a * h.h0 + (1.f - 0.5f * s2a) * udg;
+    o.hx = h.hx - k.s1n * (h.hx - rho * ux) + (1.f - 0.5f * k.s1n) * Ftx;
+    o.hy = h.hy - k.s1n * (h.hy - rho * uy) + (1.f - 0.5f * k.s1n) * Fty;
+    o.hxx = h.hxx - s2a * (h.hxx - exx) + (1.f - 0.5f * s2a) * Mxx;
+    o.hyy = h.hyy - s2a * (h.hyy - eyy) + (1.f - 0.5f * s2a) * Myy;
+    o.hxy = h.hxy - s2b * (h.hxy - exy) + (1.f - 0.5f * s2b) * Mxy;
+    o.hxyy = h.hxyy * (1.f - k.s3n);
+    o.hxxy = h.hxxy * (1.f - k.s3n);
+    o.h4 = h.h4 - s2a * (h.h4 - e4);
+    float go[9];
+    from_natural(natural_of(o, cs2, cs4), go);
+    store(g_out, 0, 0, 0, 0, go[0]);
+    store(g_out, 1, 3, 1, 0, go[1]);
+    store(g_out, 2, 4, 0, 1, go[2]);
+    store(g_out, 3, 1, -1, 0, go[3]);
+    store(g_out, 4, 2, 0, -1, go[4]);
+    store(g_out, 5, 7, 1, 1, go[5]);
+    store(g_out, 6, 8, -1, 1, go[6]);
+    store(g_out, 7, 5, -1, -1, go[7]);
+    store(g_out, 8, 6, 1, -1, go[8]);
+  }
+
+  // ---- CH collision ----
+  {
+        const float emb = k.eta * mub;
+    const float corr = k.corr_scale * (1.f - fdeg);
+    // R first moment: d_t(phi1 u) + cs2 * corr * eta grad mubar
+    const float Rx = (ph1 * ux - php * uxp) + cs2 * corr * k.eta * gmx;
+    const float Ry = (ph1 * uy - php * uyp) + cs2 * corr * k.eta * gmy;
+    float fo[9];
+    if (k.ch_fast != 0.f) {
+      // every moment but the first relaxes at rate 1, so f* = f^eq + w_i c_i . dj / cs2 with
+      // the post-collision first moment o = phi u + (1 - s1)(j - phi u) + (1 - s1/2) R
+      const float ox = ph1 * ux + (1.f - k.s1c) * (jx - ph1 * ux) + (1.f - 0.5f * k.s1c) * Rx;
+      const float oy = ph1 * uy + (1.f - k.s1c) * (jy - ph1 * uy) + (1.f - 0.5f * k.s1c) * Ry;
+      const float ic = __frcp_rn(cs2);
+      const float ax = ox * ic, ay = oy * ic;
+      fo[1] = k.wa * (emb + ax);
+      fo[3] = k.wa * (emb - ax);
+      fo[2] = k.wa * (emb + ay);
+      fo[4] = k.wa * (emb - ay);
+      fo[5] = k.we * (emb + ax + ay);
+      fo[6] = k.we * (emb - ax + ay);
+      fo[7] = k.we * (emb - ax - ay);
+      fo[8] = k.we * (emb + ax - ay);
+      // rest population closes the zeroth moment exactly
+      fo[0] = ph1 - (((fo[1] + fo[3]) + (fo[2] + fo[4])) + ((fo[5] + fo[7]) + (fo[6] + fo[8])));
+    } else {
+      // every moment enters: the populations of this node again (L2-resident)
+      float fv[9];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) fv[i] = f_in[i * pl + node];
+      Nat nf = natural(fv);
+      nf.m0 = ph1;   // zeroth moment is the phase field itself
+      const Her h = hermite(nf, cs2, cs4);
+      const float exx = cs2 * (emb - ph1);
+      Her o;
+      o.h0 = ph1;
+      o.hx = h.hx - k.s1c * (h.hx - ph1 * ux) + (1.f - 0.5f * k.s1c) * Rx;
+      o.hy = h.hy - k.s1c * (h.hy - ph1 * uy) + (1.f - 0.5f * k.s1c) * Ry;
+      o.hxx = h.hxx - k.s2ac * (h.hxx - exx);
+      o.hyy = h.hyy - k.s2ac * (h.hyy - exx);
+      o.hxy = h.hxy * (1.f - k.s2bc);
+      o.hxyy = h.hxyy * (1.f - k.s3c);
+      o.hxxy = h.hxxy * (1.f - k.s3c);
+      o.h4 = h.h4 - k.s4c * (h.h4 - cs4 * (ph1 - emb));
+      from_natural(natural_of(o, cs2, cs4), fo);
+    }
+    store(f_out, 0, 0, 0, 0, fo[0]);
+    store(f_out, 1, 3, 1, 0, fo[1]);
+    store(f_out, 2, 4, 0, 1, fo[2]);
+    store(f_out, 3, 1, -1, 0, fo[3]);
+    store(f_out, 4, 2, 0, -1, fo[4]);
+    store(f_out, 5, 7, 1, 1, fo[5]);
+    store(f_out, 6, 8, -1, 1, fo[6]);
+    store(f_out, 7, 5, -1, -1, fo[7]);
+    store(f_out, 8, 6, 1, -1, fo[8]);
+  }
+
+  // history of this step
+  h_out[node] = ph1;
+  h_out[pl + node] = ux;
+  h_out[2 * pl + node] = uy;
+  h_out[3 * pl + node] = Sx;
+  h_out[4 * pl + node] = Sy;
+  if (OBS) {
+    a.p_out[(long long)b * plane + node] = p;
+    const float u2 = ux * ux + uy * uy;
+    if (!(u2 <= 0.25f) || !(fabsf(ph1) < 1e30f)) atomicOr(a.flag, 1u);
+  }
+}
 
 // One CTA's work: columns x0 .. x0+127 and rows ys .. ys+strip-1 of instance b.
 // PER: both axes periodic (known at compile time), so no push can meet a wall
@@ -443,15 +673,9 @@ __device__ __forceinline__ void step_tile(const StepArgs& a, StepSmem<D, GT>& S,
       float v[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) v[i] = slot.rows[i][col];
-      float sum = v[0];
-#pragma unroll
-      for (int i = 1; i < 9; ++i) sum += v[i];
-      S.phi1[sp][c] = sum;
+      S.phi1[sp][c] = phase_sum(v);
       S.phi0[sp][c] = slot.rows[9][col];
-      if (own) {
-        jx = (v[1] - v[3]) + (v[5] - v[6]) - (v[7] - v[8]);
-        jy = (v[2] - v[4]) + (v[5] + v[6]) - (v[7] + v[8]);
-      }
+      if (own) first_moment(v, jx, jy);
     };
     one(t + 2, true);
     // the four halo columns 0, 1, BX+2, BX+3, one per warp
@@ -469,25 +693,24 @@ __device__ __forceinline__ void step_tile(const StepArgs& a, StepSmem<D, GT>& S,
     const float* A0m = S.phi0[cm];
     const float* A0p = S.phi0[cp];
     const float* A0q = S.phi0[cq];
-    auto one = [&](int s, bool own) {
+    auto one = [&](auto edge, int s) {
       const int xl = x0 - 1 + s;
       if (xl > nx) return;
       const int c = s + 1;
       const P9 v1{A1p[c], A1p[c + 1], A1q[c], A1p[c - 1], A1m[c], A1q[c + 1], A1q[c - 1], A1m[c - 1], A1m[c + 1]};
       const P9 v0{A0p[c], A0p[c + 1], A0q[c], A0p[c - 1], A0m[c], A0q[c + 1], A0q[c - 1], A0m[c - 1], A0m[c + 1]};
-      float mu0, mu1, mu2;
-      chem_pot(k, v0.c, v1.c, iso_lap(v0), iso_lap(v1), mu0, mu1, mu2);
-      S.mub[sm][s] = mubar1_of(k, mu0, mu1, mu2);
+      float e02, e12;
+      mu_point<decltype(edge)::value>(k, v0, v1, S.mub[sm][s], e02, e12);
       const int col = s + PAD - 1;
-      S.acorr[sm][s] = slot.rows[3][col] * slot.rows[2][col] - slot.rows[1][col] * slot.rows[4][col];
-      if (own) {
-        d02 = mu0 - mu2;
-        d12 = mu1 - mu2;
+      S.acorr[sm][s] = correction_product(slot.rows[3][col], slot.rows[2][col], slot.rows[1][col], slot.rows[4][col]);
+      if (!decltype(edge)::value) {
+        d02 = e02;
+        d12 = e12;
       }
     };
-    one(t + 1, true);                 // this thread's own column
-    if (t == 64) one(0, false);       // halo columns, on warps 2 and 3
-    if (t == 96) one(BX + 1, false);
+    one(std::false_type(), t + 1);            // this thread's own column
+    if (t == 64) one(std::true_type(), 0);    // halo columns, on warps 2 and 3
+    if (t == 96) one(std::true_type(), BX + 1);
   };
 
   // The sweep starts four iterations early: iterations ys-4 .. ys-1 only run
@@ -517,8 +740,6 @@ __device__ __forceinline__ void step_tile(const StepArgs& a, StepSmem<D, GT>& S,
       const HRow& hs = S.h[ring(y, D + 2)];
       const int c = t + 2, s = t + 1, col = t + PAD;
       const int node = y * nx + x;         // instance-relative, < 2^31 (checked at creation)
-      const int pl = (int)plane;
-      const float cs2 = k.cs2, cs4 = k.cs4;
       float g[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) g[i] = g_load(gs.rows[i][t + gpad<GT>()], k);
@@ -542,175 +763,8 @@ __device__ __forceinline__ void step_tile(const StepArgs& a, StepSmem<D, GT>& S,
       const P9 vm{M0[0], M0[1], Mp[0], M0[-1], Mm[0], Mp[1], Mp[-1], Mm[-1], Mm[1]};
       const P9 va{0.f, A0[1], Ap[0], A0[-1], Am[0], Ap[1], Ap[-1], Am[-1], Am[1]};
 
-      const float ph1 = v1.c, ph0 = v0.c, ph2 = 1.f - ph0 - ph1;
-      float g1x, g1y, g0x, g0y, gmx, gmy, dAx, dAy;
-      iso_grad(v1, g1x, g1y);
-      iso_grad(v0, g0x, g0y);
-      iso_grad(vm, gmx, gmy);
-      iso_grad(va, dAx, dAy);
-      const float mub = vm.c;
-
-      // degenerate mobility, mass flux S (frozen phi0), mixture properties
-      const float fdeg = ph1 * (1.f - ph1) * (1.f - ph0);
-      const float mob = k.M_cst + k.M_deg * fdeg;
-      const float sfac = (k.rho1 - k.rho2) * mob * k.inv_gam1;
-      const float Sx = sfac * gmx, Sy = sfac * gmy;
-      const float rho = k.rho0 * ph0 + k.rho1 * ph1 + k.rho2 * ph2;
-      const float grx = (k.rho0 - k.rho2) * g0x + (k.rho1 - k.rho2) * g1x;
-      const float gry = (k.rho0 - k.rho2) * g0y + (k.rho1 - k.rho2) * g1y;
-      const float muv = k.mu0 * ph0 + k.mu1 * ph1 + k.mu2 * ph2;
-
-      // F = F_s + F_b + F_c, F_s = (mu0 - mu2) grad phi0 + (mu1 - mu2) grad phi1
-      const float one_m0 = 1.f - ph0;
-      const float Fx = d02 * g0x + d12 * g1x + one_m0 * k.bx - 0.5f * dAy;
-      const float Fy = d02 * g0y + d12 * g1y + one_m0 * k.by + 0.5f * dAx;
-
-      // NS moments, velocity with the solid penalisation force
-      const Nat ng = natural(g);
-      const float inv_rho = __frcp_rn(rho);
-      const float usx = (ng.mx + 0.5f * Fx) * inv_rho;
-      const float usy = (ng.my + 0.5f * Fy) * inv_rho;
-      const float damp = 1.f - 0.5f * ph0;
-      const float ux = usx * damp, uy = usy * damp;
-      const float Ftx = Fx - ph0 * rho * usx, Fty = Fy - ph0 * rho * usy;
-
-      // local viscous rates (s0 = s4 = s2a)
-      const float om = fmaxf(one_m0, kOneMinusPhi0Floor);
-      // 1/s2a = 1/2 + mu / (rho (1 - phi0) a2a), likewise s2b; IEEE-rounded reciprocals
-      const float nu_e = muv * __frcp_rn(rho * om);
-      const float inv_s2a = 0.5f + nu_e * k.ia2a;
-      const float s2a = __frcp_rn(inv_s2a);
-      const float s2b = __frcp_rn(0.5f + nu_e * k.ia2b);
-
-      // pressure
-      const float udg = ux * grx + uy * gry;
-      const float q = (rho * ux - Sx) * ux + (rho * uy - Sy) * uy;
-      const float rhop = k.rho0 * ph0 + k.rho1 * php + k.rho2 * (1.f - ph0 - php);
-      const float qp = (rhop * uxp - Sxp) * uxp + (rhop * uyp - Syp) * uyp;
-      const float H = k.Kp * ((k.h0 - k.h2) * inv_s2a + k.h3);
-      const float sum_nz = ng.m0 - g[0];
-      const float p = k.pf * (sum_nz + (0.5f + H) * udg - k.wq * q + 0.5f * k.Kp * (q - qp));
-
-      // destinations of the nine pushes without branches: per axis and sign the
-      // neighbour's offset (periodic wrap folded in) and whether a wall reflects
-      const bool wxp = !PER && x + 1 >= nx && !per_x, wxm = !PER && x == 0 && !per_x;
-      const bool wyp = !PER && y + 1 >= ny && !per_y, wym = !PER && y == 0 && !per_y;
-      const int oxp = x + 1 < nx ? 1 : 1 - nx, oxm = x > 0 ? -1 : nx - 1;
-      const int oyp = y + 1 < ny ? nx : nx - pl, oym = y > 0 ? -nx : pl - nx;
-      auto store = [&](auto* __restrict__ out, int i, int io, int cx, int cy, float v) {
-        int off = 0;
-        bool bb = false;
-        if (cx) { off += cx > 0 ? oxp : oxm; bb = bb || (cx > 0 ? wxp : wxm); }
-        if (cy) { off += cy > 0 ? oyp : oym; bb = bb || (cy > 0 ? wyp : wym); }
-        g_store(out + (bb ? io * pl + node : i * pl + node + off), v, k);
-      };
-
-      // ---- NS collision in Hermite space ----
-      {
-        const Her h = hermite(ng, cs2, cs4);
-        const float exx = p + rho * ux * ux - Sx * ux;
-        const float eyy = p + rho * uy * uy - Sy * uy;
-        const float exy = rho * ux * uy - 0.5f * (Sx * uy + ux * Sy);
-        const float e4 = -cs2 * p;
-        const float dSxx = Sx * ux - Sxp * uxp;
-        const float dSyy = Sy * uy - Syp * uyp;
-        const float dSxy = 0.5f * (Sx * uy + ux * Sy) - 0.5f * (Sxp * uyp + uxp * Syp);
-        const float iso = (1.f - 3.f * cs2) * udg;
-        const float Mxx = 2.f * ux * Fx - dSxx + 2.f * cs2 * ux * grx + iso;
-        const float Myy = 2.f * uy * Fy - dSyy + 2.f * cs2 * uy * gry + iso;
-        const float Mxy = ux * Fy + Fx * uy - dSxy + cs2 * (ux * gry + grx * uy);
-        Her o;
-        o.h0 = h.h0 - s2a * h.h0 + (1.f - 0.5f * s2a) * udg;
-        o.hx = h.hx - k.s1n * (h.hx - rho * ux) + (1.f - 0.5f * k.s1n) * Ftx;
-        o.hy = h.hy - k.s1n * (h.hy - rho * uy) + (1.f - 0.5f * k.s1n) * Fty;
-        o.hxx = h.hxx - s2a * (h.hxx - exx) + (1.f - 0.5f * s2a) * Mxx;
-        o.hyy = h.hyy - s2a * (h.hyy - eyy) + (1.f - 0.5f * s2a) * Myy;
-        o.hxy = h.hxy - s2b * (h.hxy - exy) + (1.f - 0.5f * s2b) * Mxy;
-        o.hxyy = h.hxyy * (1.f - k.s3n);
-        o.hxxy = h.hxxy * (1.f - k.s3n);
-        o.h4 = h.h4 - s2a * (h.h4 - e4);
-        float go[9];
-        from_natural(natural_of(o, cs2, cs4), go);
-        store(g_out, 0, 0, 0, 0, go[0]);
-        store(g_out, 1, 3, 1, 0, go[1]);
-        store(g_out, 2, 4, 0, 1, go[2]);
-        store(g_out, 3, 1, -1, 0, go[3]);
-        store(g_out, 4, 2, 0, -1, go[4]);
-        store(g_out, 5, 7, 1, 1, go[5]);
-        store(g_out, 6, 8, -1, 1, go[6]);
-        store(g_out, 7, 5, -1, -1, go[7]);
-        store(g_out, 8, 6, 1, -1, go[8]);
-      }
-
-      // ---- CH collision ----
-      {
-        const float jx = jx0, jy = jy0;
-        const float emb = k.eta * mub;
-        const float corr = k.corr_scale * (1.f - fdeg);
-        // R first moment: d_t(phi1 u) + cs2 * corr * eta grad mubar
-        const float Rx = (ph1 * ux - php * uxp) + cs2 * corr * k.eta * gmx;
-        const float Ry = (ph1 * uy - php * uyp) + cs2 * corr * k.eta * gmy;
-        float fo[9];
-        if (k.ch_fast != 0.f) {
-          // every moment but the first relaxes at rate 1, so f* = f^eq + w_i c_i . dj / cs2 with
-          // the post-collision first moment o = phi u + (1 - s1)(j - phi u) + (1 - s1/2) R
-          const float ox = ph1 * ux + (1.f - k.s1c) * (jx - ph1 * ux) + (1.f - 0.5f * k.s1c) * Rx;
-          const float oy = ph1 * uy + (1.f - k.s1c) * (jy - ph1 * uy) + (1.f - 0.5f * k.s1c) * Ry;
-          const float ic = __frcp_rn(cs2);
-          const float ax = ox * ic, ay = oy * ic;
-          fo[1] = k.wa * (emb + ax);
-          fo[3] = k.wa * (emb - ax);
-          fo[2] = k.wa * (emb + ay);
-          fo[4] = k.wa * (emb - ay);
-          fo[5] = k.we * (emb + ax + ay);
-          fo[6] = k.we * (emb - ax + ay);
-          fo[7] = k.we * (emb - ax - ay);
-          fo[8] = k.we * (emb + ax - ay);
-          // rest population closes the zeroth moment exactly
-          fo[0] = ph1 - (((fo[1] + fo[3]) + (fo[2] + fo[4])) + ((fo[5] + fo[7]) + (fo[6] + fo[8])));
-        } else {
-          // every moment enters: the populations of this node again (L2-resident)
-          float fv[9];
-#pragma unroll
-          for (int i = 0; i < 9; ++i) fv[i] = f_in[i * pl + node];
-          Nat nf = natural(fv);
-          nf.m0 = ph1;   // zeroth moment is the phase field itself
-          const Her h = hermite(nf, cs2, cs4);
-          const float exx = cs2 * (emb - ph1);
-          Her o;
-          o.h0 = ph1;
-          o.hx = h.hx - k.s1c * (h.hx - ph1 * ux) + (1.f - 0.5f * k.s1c) * Rx;
-          o.hy = h.hy - k.s1c * (h.hy - ph1 * uy) + (1.f - 0.5f * k.s1c) * Ry;
-          o.hxx = h.hxx - k.s2ac * (h.hxx - exx);
-          o.hyy = h.hyy - k.s2ac * (h.hyy - exx);
-          o.hxy = h.hxy * (1.f - k.s2bc);
-          o.hxyy = h.hxyy * (1.f - k.s3c);
-          o.hxxy = h.hxxy * (1.f - k.s3c);
-          o.h4 = h.h4 - k.s4c * (h.h4 - cs4 * (ph1 - emb));
-          from_natural(natural_of(o, cs2, cs4), fo);
-        }
-        store(f_out, 0, 0, 0, 0, fo[0]);
-        store(f_out, 1, 3, 1, 0, fo[1]);
-        store(f_out, 2, 4, 0, 1, fo[2]);
-        store(f_out, 3, 1, -1, 0, fo[3]);
-        store(f_out, 4, 2, 0, -1, fo[4]);
-        store(f_out, 5, 7, 1, 1, fo[5]);
-        store(f_out, 6, 8, -1, 1, fo[6]);
-        store(f_out, 7, 5, -1, -1, fo[7]);
-        store(f_out, 8, 6, 1, -1, fo[8]);
-      }
-
-      // history of this step
-      h_out[node] = ph1;
-      h_out[pl + node] = ux;
-      h_out[2 * pl + node] = uy;
-      h_out[3 * pl + node] = Sx;
-      h_out[4 * pl + node] = Sy;
-      if (OBS) {
-        a.p_out[(long long)b * plane + node] = p;
-        const float u2 = ux * ux + uy * uy;
-        if (!(u2 <= 0.25f) || !(fabsf(ph1) < 1e30f)) atomicOr(a.flag, 1u);
-      }
+      collide_node<OBS, GT, PER>(a, k, b, node, x, y, v1, v0, vm, va, d02, d12, jx0, jy0, g, php, uxp, uyp, Sxp, Syp, f_in,
+                                 f_out, g_out, h_out);
     }
     d02 = n02;
     d12 = n12;
@@ -720,6 +774,153 @@ __device__ __forceinline__ void step_tile(const StepArgs& a, StepSmem<D, GT>& S,
     mm = m0; m0 = mp; mp = inc_mod(mp, RM);
   }
   cp_wait<0>();
+}
+
+// ---------------------------------------------------------------------------
+// Fused step on small lattices: a CTA owns 32 x TY nodes, one per thread, and makes the whole step in three stages
+// with two barriers.  Every load is issued at the start (own populations, history and phi0, and the points of the
+// halo that the thread takes on: two halo nodes of phi, one of mubar_1), so a step costs one memory latency and two
+// barriers, where the sweep above costs three barriers and a copy's latency per row of its strip.  The price is the
+// halo: (36 / 32)((TY + 4) / TY) sums of nine populations per node instead of 132 / 128.
+// With programmatic launch a step's CTAs start while the previous step drains, load the constants and phi0 (which no
+// step writes) and wait for it there.
+// Measured (GB300, us per step, replayed graphs; the sweep at its best strip): 128 x 64 with y walls 2.9 against 11.3,
+// 483 x 127 with walls 4.9 against 11.0, 512^2 11.1 against 18.9, 5 x 256^2 with FP16 populations 14.4 against 22.4,
+// 1024^2 49 against 52, 5 x 1024^2 229 against 212.  TY = 4 is faster while its CTAs stay below four per SM (256^2: 5.4
+// against 5.8 us for TY = 8, 512^2: 12.4 against 11.1); TY = 16 is slower everywhere.
+// ---------------------------------------------------------------------------
+constexpr int TX = 32;
+
+template <bool OBS, typename GT, bool PER, int TY>
+__global__ void __launch_bounds__(TX * TY) d2q9_tile(const StepArgs a) {
+  constexpr int NT = TX * TY, W2 = TX + 4, W1 = TX + 2;
+  constexpr int HALO2 = 4 * W2 + 4 * TY, HALO1 = 2 * W1 + 2 * TY;   // points around the owned ones, two and one deep
+  static_assert(HALO1 <= NT, "one mubar_1 halo point a thread");
+  __shared__ float phi1[TY + 4][W2], phi0[TY + 4][W2], mub[TY + 2][W1], cor[TY + 2][W1];
+  __shared__ InstanceConsts k;
+  const int t = threadIdx.x, tx = t % TX, ty = t / TX;
+  const int nx = a.nx, ny = a.ny, per_x = a.per_x, per_y = a.per_y;
+  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, b = blockIdx.z;
+  const int pl = (int)a.nodes;
+  const float* __restrict__ f_in = a.f_in + (long long)b * 9 * pl;
+  const GT* __restrict__ g_in = static_cast<const GT*>(a.g_in) + (long long)b * 9 * pl;
+  const float* __restrict__ p0_in = a.phi0 + (long long)b * pl;
+  const float* __restrict__ h_in = a.hist_in + (long long)b * 5 * pl;
+  const int x = x0 + tx, y = y0 + ty;
+
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int i = t; i < (int)(sizeof(InstanceConsts) / 4); i += NT)
+    reinterpret_cast<float*>(&k)[i] = reinterpret_cast<const float*>(a.consts + b)[i];
+
+  // node index of tile position (px, py) relative to (x0, y0), -1 beyond what the last real node needs: `deep` nodes
+  // past the lattice, wrapped or mirrored
+  auto at = [&](int px, int py, int deep) {
+    const int xl = x0 + px, yl = y0 + py;
+    if (xl >= nx + deep || yl >= ny + deep) return -1;
+    return wrap_or_mirror_row(yl, ny, per_y) * nx + wrap_or_mirror_row(xl, nx, per_x);
+  };
+  const int own2 = at(tx, ty, 2);
+  constexpr int ROUNDS = (HALO2 + NT - 1) / NT;
+  int hx[ROUNDS], hy[ROUNDS], hn[ROUNDS];
+  float h0[ROUNDS];
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) {
+    const int p = t + r * NT;
+    if (p < 4 * W2) {                      // two rows below, two above
+      const int row = p / W2;
+      hx[r] = p - row * W2 - 2;
+      hy[r] = row < 2 ? row - 2 : TY + row - 2;
+    } else {
+      const int q = p - 4 * W2, col = q & 3;
+      hx[r] = col < 2 ? col - 2 : TX + col - 2;
+      hy[r] = q >> 2;
+    }
+    hn[r] = p < HALO2 ? at(hx[r], hy[r], 2) : -1;
+    h0[r] = hn[r] >= 0 ? p0_in[hn[r]] : 0.f;
+  }
+  // the mubar_1 halo point of this thread
+  int mx = 0, my = 0, mn = -1;
+  if (t < HALO1) {
+    if (t < 2 * W1) {
+      const int row = t / W1;
+      mx = t - row * W1 - 1;
+      my = row == 0 ? -1 : TY;
+    } else {
+      const int q = t - 2 * W1;
+      mx = (q & 1) ? TX : -1;
+      my = q >> 1;
+    }
+    mn = at(mx, my, 1);
+  }
+  const float own0 = own2 >= 0 ? p0_in[own2] : 0.f;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  // every load of what the previous step wrote
+  float f[9], hf[ROUNDS][9], g[9], hist[5], mh[4];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) f[i] = own2 >= 0 ? f_in[i * pl + own2] : 0.f;
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r)
+#pragma unroll
+    for (int i = 0; i < 9; ++i) hf[r][i] = hn[r] >= 0 ? f_in[i * pl + hn[r]] : 0.f;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) hist[i] = own2 >= 0 ? h_in[i * pl + own2] : 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) mh[i] = mn >= 0 ? h_in[(i + 1) * pl + mn] : 0.f;
+  GT graw[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) graw[i] = own2 >= 0 ? g_in[i * pl + own2] : GT(0.f);
+
+  // stage 1: phi1 on the tile with two halo nodes
+  float jx, jy;
+  phi1[ty + 2][tx + 2] = phase_sum(f);
+  phi0[ty + 2][tx + 2] = own0;
+  first_moment(f, jx, jy);
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r)
+    if (hn[r] >= 0) {
+      phi1[hy[r] + 2][hx[r] + 2] = phase_sum(hf[r]);
+      phi0[hy[r] + 2][hx[r] + 2] = h0[r];
+    }
+  __syncthreads();
+
+  // stage 2: mubar_1 and the correction-force product on the tile with one halo node
+  auto hood = [&](const float (*v)[W2], int px, int py) {
+    const float *m = v[py + 1] + px + 2, *c = v[py + 2] + px + 2, *q = v[py + 3] + px + 2;
+    return P9{c[0], c[1], q[0], c[-1], m[0], q[1], q[-1], m[-1], m[1]};
+  };
+  float d02 = 0.f, d12 = 0.f;
+  auto stage2 = [&](auto edge, int px, int py, float ux, float uy, float sx, float sy, float& e02, float& e12) {
+    mu_point<decltype(edge)::value>(k, hood(phi0, px, py), hood(phi1, px, py), mub[py + 1][px + 1], e02, e12);
+    cor[py + 1][px + 1] = correction_product(sx, uy, ux, sy);
+  };
+  // column px is the halo column of a whole 128-column tile of the sweep: left of its start, or right of its end
+  auto edge = [&](int px) { return px < 0 ? x0 % BX == 0 : (px >= TX && (x0 + px) % BX == 0); };
+  using Edge = std::true_type;
+  using Inner = std::false_type;
+  if (x <= nx && y <= ny) stage2(Inner(), tx, ty, hist[1], hist[2], hist[3], hist[4], d02, d12);
+  if (mn >= 0) {
+    float e02, e12;
+    if (edge(mx)) stage2(Edge(), mx, my, mh[0], mh[1], mh[2], mh[3], e02, e12);
+    else stage2(Inner(), mx, my, mh[0], mh[1], mh[2], mh[3], e02, e12);
+  }
+  __syncthreads();
+
+  // stage 3
+  if (x >= nx || y >= ny) return;
+  const P9 v1 = hood(phi1, tx, ty), v0 = hood(phi0, tx, ty);
+  auto hood1 = [&](const float (*v)[W1]) {
+    const float *m = v[ty] + tx + 1, *c = v[ty + 1] + tx + 1, *q = v[ty + 2] + tx + 1;
+    return P9{c[0], c[1], q[0], c[-1], m[0], q[1], q[-1], m[-1], m[1]};
+  };
+  const P9 vm = hood1(mub);
+  P9 va = hood1(cor);
+  va.c = 0.f;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) g[i] = g_load(graw[i], k);
+  collide_node<OBS, GT, PER>(a, k, b, y * nx + x, x, y, v1, v0, vm, va, d02, d12, jx, jy, g, hist[0], hist[1], hist[2],
+                             hist[3], hist[4], f_in, a.f_out + (long long)b * 9 * pl,
+                             static_cast<GT*>(a.g_out) + (long long)b * 9 * pl, a.hist_out + (long long)b * 5 * pl);
 }
 
 // one tile per CTA: grid (column tiles, row strips, instances)
@@ -819,7 +1020,31 @@ cudaError_t launch_typed(const StepArgs& a, int nbatch, bool observe, cudaStream
   }
 }
 
+template <typename GT, bool PER, int TY>
+cudaError_t launch_tile(const StepArgs& a, int nbatch, bool observe, cudaStream_t s) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, nbatch);
+  cfg.blockDim = dim3(TX * TY);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return observe ? cudaLaunchKernelEx(&cfg, d2q9_tile<true, GT, PER, TY>, a)
+                 : cudaLaunchKernelEx(&cfg, d2q9_tile<false, GT, PER, TY>, a);
+}
+
+template <typename GT>
+cudaError_t launch_tile(const StepArgs& a, int nbatch, bool observe, cudaStream_t s) {
+  const bool per = a.per_x && a.per_y;
+  if (a.tile == 4)
+    return per ? launch_tile<GT, true, 4>(a, nbatch, observe, s) : launch_tile<GT, false, 4>(a, nbatch, observe, s);
+  return per ? launch_tile<GT, true, 8>(a, nbatch, observe, s) : launch_tile<GT, false, 8>(a, nbatch, observe, s);
+}
+
 cudaError_t launch_d2q9_step(const StepArgs& a, int nbatch, bool observe, cudaStream_t s) {
+  if (a.tile) return a.g_half ? launch_tile<__half>(a, nbatch, observe, s) : launch_tile<float>(a, nbatch, observe, s);
   return a.g_half ? launch_typed<__half>(a, nbatch, observe, s) : launch_typed<float>(a, nbatch, observe, s);
 }
 

@@ -261,9 +261,11 @@ __global__ void d3q19_init(const float* __restrict__ phi0_all, const float* __re
       float* f = f_all + (long long)b * QL * nodes;
       GT* g = g_all + (long long)b * QL * nodes;
       float* h = hist_all + (long long)b * NH * nodes;
+      // the constants before the stores, which could alias them as far as the compiler knows
+      const float fa = k.wa * emb, fe = k.we * emb;
       f[node] = c1 + (k.w0 - 1.f) * emb;
 #pragma unroll
-      for (int i = 1; i < QL; ++i) f[(long long)i * nodes + node] = (i < 7 ? k.wa : k.we) * emb;
+      for (int i = 1; i < QL; ++i) f[(long long)i * nodes + node] = i < 7 ? fa : fe;
 #pragma unroll
       for (int i = 0; i < QL; ++i) g[(long long)i * nodes + node] = GT(0.f);
       h[node] = c1;

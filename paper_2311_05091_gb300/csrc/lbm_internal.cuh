@@ -80,6 +80,7 @@ struct StepArgs {
   int strip;              // rows (2D) or planes (3D) per CTA
   int depth;              // rows of asynchronous copies kept in flight (1..3)
   long long nodes;        // nodes per instance
+  int tile;               // D2Q9: rows (4 or 8) of the small-lattice kernel's tiles, 0: the sweep
   int g_half;             // NS populations stored as FP16
   int q;                  // lattice directions (9, 15 or 19)
   int wait_polls;         // polls of a bounded tile-load wait before it gives up (3D pipelined kernel)
