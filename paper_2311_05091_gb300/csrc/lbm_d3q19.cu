@@ -1001,11 +1001,7 @@ __device__ __forceinline__ void tma_load4(void* dst, const CUtensorMap* map, int
       : "memory");
 }
 
-// VEC: rows on 16 bytes (nx % 4 == 0; FP16 g: 8).  Otherwise neither the TMA tiles nor 16-byte chunks apply, and the
-// same pipeline runs on 4-byte asynchronous copies: each thread copies the owned values of its own column, the halo
-// chunks go element by element.  Measured on 117 x 97 x 75 (D3Q15, walls in z, mass flux): VEC_US per step against 138
-// for the generic form with its synchronous loads.
-template <int QL, bool OBS, typename GT, bool SZ = false, bool PER = false, bool VEC = true, int TYP = kPipeTY>
+template <int QL, bool OBS, typename GT, bool SZ = false, bool PER = false, int TYP = kPipeTY>
 __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
     d3q19_step_pipe(const StepArgs a, const __grid_constant__ TmaMaps maps) {
   using Smem = PipeSmem3<QL, GT, TYP>;
@@ -1054,12 +1050,6 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
     off = 0;
     if (ylog > ymax || xs > xmax) return;
     const int yr = wrap_or_mirror(ylog, ny, per_y) * nx;
-    if (!VEC) {
-      // inside the row: four consecutive words; else the row's start, columns folded back word by word
-      mode = xs >= 0 && xs + 3 < nx ? 0 : 2;
-      off = mode == 0 ? yr + xs : yr;
-      return;
-    }
     if (xs >= 0 && xs < nx) {
       mode = 0;
       off = yr + xs;
@@ -1090,16 +1080,8 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
     hc_dst[m] = r * PW + 4 * kk;
     hc_arr[m] = arr;
   }
-  // chunk columns of `dst` start at lattice column x0 - 4 + kk, kk its offset in the tile row
-  auto copy_chunk = [&](float* dst, const float* src, int mode, int kk, int xmax) {
-    if (!VEC) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int xl = x0 - 4 + kk + e;
-        if (mode == 0) cp4(dst + e, src + e);
-        else if (xl >= -2 && xl <= xmax) cp4(dst + e, src + wrap_or_mirror(xl, nx, per_x));
-      }
-    } else if (mode == 0) {
+  auto copy_chunk = [&](float* dst, const float* src, int mode) {
+    if (mode == 0) {
       cp16(dst, src);
     } else if (mode == 1) {
       cp4(dst, src);
@@ -1112,7 +1094,7 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
     if (pc_mode < 0) return;
     const int zo = wrap_or_mirror(zl, nz, per_z) * plane;
     float* base = (t / (PR2 * 10) == 0 ? S.phi1 : S.phi0)[ring(zl, RP5)];
-    copy_chunk(base + pc_dst, pc_src + zo + pc_off, pc_mode, pc_dst % PW, nx + 1);
+    copy_chunk(base + pc_dst, pc_src + zo + pc_off, pc_mode);
   };
   auto issue_hist = [&](int zl) {
     const int zo = wrap_or_mirror(zl, nz, per_z) * plane;
@@ -1120,31 +1102,11 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       if (hc_mode[m] < 0) continue;
-      copy_chunk(&S.hus[sl][hc_arr[m]][hc_dst[m]], h_in + (hc_arr[m] + 1) * nodes + zo + hc_off[m], hc_mode[m],
-                 hc_dst[m] % PW, nx);
+      copy_chunk(&S.hus[sl][hc_arr[m]][hc_dst[m]], h_in + (hc_arr[m] + 1) * nodes + zo + hc_off[m], hc_mode[m]);
     }
   };
   // The owned tiles of plane z complete one phase of the barrier: g into its slot of the two-plane ring
   // (armed with the bytes of all three tiles), then j and the history into their single slot.
-  // !VEC: the owned values of this thread's column by 4-byte copies instead
-  const int x = x0 + tx, y = y0 + ty;
-  const bool own = x < nx && y < ny;
-  const float* __restrict__ g_in4 = static_cast<const float*>(a.g_in) + (long long)b * QL * nodes;
-  const float* __restrict__ j_in4 = a.mom + (long long)b * 3 * nodes;
-  auto copy_own_g = [&](int z) {
-    if (!own) return;
-    const int node = z * plane + y * nx + x;
-#pragma unroll
-    for (int i = 0; i < QL; ++i) cp4(reinterpret_cast<float*>(&S.gown[z & 1][i][t]), g_in4 + i * nodes + node);
-  };
-  auto copy_own_jh = [&](int z) {
-    if (!own) return;
-    const int node = z * plane + y * nx + x;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) cp4(&S.own[i][t], j_in4 + i * nodes + node);
-#pragma unroll
-    for (int i = 0; i < NH; ++i) cp4(&S.own[3 + i][t], h_in + i * nodes + node);
-  };
   auto issue_own_g = [&](int z) {   // one thread
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     bar_expect(&S.bar, kOwnBytes);
@@ -1213,10 +1175,7 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   __syncthreads();   // constants and barrier visible
-  if constexpr (!VEC) {
-    copy_own_g(zs);
-    copy_own_jh(zs);
-  } else if (t == 0) {
+  if (t == 0) {
     issue_own_g(zs);
     issue_own_jh(zs);
   }
@@ -1237,6 +1196,8 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
   issue_hist(zs + 1);
   cp_commit();
 
+  const int x = x0 + tx, y = y0 + ty;
+  const bool own = x < nx && y < ny;
   bool ok = true;
   unsigned pending = 0;
   for (int z = zs; z < ze; ++z) {
@@ -1245,18 +1206,14 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
     // every thread records the phase it waits on: after a block-wide give-up, the drain below waits on that
     // load (immediately satisfied for threads that saw it land) and not on the next, never-issued phase
     pending = parity;
-    if (VEC && !bar_wait(&S.bar, parity, a.wait_polls)) ok = false;   // owned planes of z
+    if (!bar_wait(&S.bar, parity, a.wait_polls)) ok = false;   // owned planes of z
     if (!__syncthreads_and(ok)) {
       if (t == 0) atomicOr(o.flag, 2u);
       ok = false;
       break;
     }
     // the g slot of z+1 held z-1, whose node updates are done
-    if constexpr (!VEC) {
-      if (z + 1 < ze) copy_own_g(z + 1);
-    } else if (t == 0 && z + 1 < ze) {
-      issue_own_g(z + 1);
-    }
+    if (t == 0 && z + 1 < ze) issue_own_g(z + 1);
     if (z + 3 <= ze + 1) issue_phi(z + 3);
     if (z + 2 <= ze) issue_hist(z + 2);
     cp_commit();
@@ -1278,13 +1235,8 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
     in.spz = S.own[9][t];
     in.d02 = S.dmu[z & 1][0][t];
     in.d12 = S.dmu[z & 1][1][t];
-    if constexpr (!VEC) {           // the slot's values of a column belong to its thread
-      if (z + 1 < ze) copy_own_jh(z + 1);
-      cp_commit();
-    } else {
-      __syncthreads();
-      if (t == 0 && z + 1 < ze) issue_own_jh(z + 1);
-    }
+    __syncthreads();
+    if (t == 0 && z + 1 < ze) issue_own_jh(z + 1);
     if (!own) continue;
 
     Rings R;
@@ -1310,7 +1262,7 @@ __global__ void __launch_bounds__(TX * TYP, TYP <= 8 ? 2 : 1)
   // leave no copy in flight: asynchronous copies, and a TMA load issued for a plane not processed
   cp_wait_all();
   // one more bounded wait, at the default limit, for the TMA load that was late
-  if (VEC && !ok) (void)bar_wait(&S.bar, pending, kWaitPollsDefault);
+  if (!ok) (void)bar_wait(&S.bar, pending, kWaitPollsDefault);
 }
 
 }  // namespace
@@ -1383,28 +1335,6 @@ cudaError_t launch_step_q(const StepArgs& a, int nbatch, bool observe, cudaStrea
   const int ntx = (a.nx + TX - 1) / TX;
   const int nstrips = (a.nz + a.strip - 1) / a.strip;
   dim3 grid(ntx * nstrips, (a.ny + TY - 1) / TY, nbatch);
-  if constexpr (std::is_same<GT, float>::value) {
-    if (!maps && a.depth != 1) {    // rows not on 16 bytes: the pipeline on 4-byte copies
-      const TmaMaps m{};
-      const size_t smem = sizeof(PipeSmem3<QL, GT, kPipeTY>);
-      constexpr int NTP = TX * kPipeTY;
-      grid.y = (a.ny + kPipeTY - 1) / kPipeTY;
-      static std::atomic<unsigned long long> configured{0};
-      e = smem_opt_in(configured, smem, d3q19_step_pipe<QL, true, GT, false, false, false>,
-                      d3q19_step_pipe<QL, false, GT, false, false, false>,
-                      d3q19_step_pipe<QL, true, GT, true, false, false>,
-                      d3q19_step_pipe<QL, false, GT, true, false, false>);
-      if (e != cudaSuccess) return e;
-      if (a.s_zero) {
-        if (observe) d3q19_step_pipe<QL, true, GT, true, false, false><<<grid, NTP, smem, s>>>(a, m);
-        else d3q19_step_pipe<QL, false, GT, true, false, false><<<grid, NTP, smem, s>>>(a, m);
-      } else {
-        if (observe) d3q19_step_pipe<QL, true, GT, false, false, false><<<grid, NTP, smem, s>>>(a, m);
-        else d3q19_step_pipe<QL, false, GT, false, false, false><<<grid, NTP, smem, s>>>(a, m);
-      }
-      return cudaGetLastError();
-    }
-  }
   if (maps) {
     TmaMaps m;
     memcpy(&m, maps, sizeof m);
