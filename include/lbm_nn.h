@@ -98,7 +98,8 @@ int lbm_nn_to_bf16(const float* a, void* b, long long n, void* stream);
  * lambda = clamp((sum phi1 - sum field) / sum b, -1, 1), which restores the
  * phase mass of the initial field (sum phi1) while every value stays in
  * [0, hi] (for |lambda| <= 1 the correction is monotone with fixed points 0
- * and hi).  work: at least 192 n doubles. */
+ * and hi).  work: at least 192 n doubles; with 384 n a pass takes one launch
+ * instead of two, with the same result. */
 int lbm_nn_project(const float* out, int cpad, const float* phi0, const float* phi1, float* field, double* work,
                    long long work_len, int n, int h, int w, void* stream);
 

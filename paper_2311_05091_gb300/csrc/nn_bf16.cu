@@ -997,30 +997,67 @@ __global__ void add(float* z, const float* x, const float* y, float a, long long
   if (i < n) z[i] = x[i] + a * y[i];
 }
 
-// input tensor [p][16]: phi0, phi1, cos theta of the image, zeros
+// input tensor [p][16]: phi0, phi1, cos theta of the image, zeros.  Bound by its writes (64 bytes a node), so they must
+// be whole lines: a warp's 32 nodes are one run of 2 KB, which it writes as consecutive float4 with the values taken from
+// the lanes that loaded them (16 images of 256^2: 12 us, where a thread that wrote its own node took 70).  V4 needs x on
+// 16 bytes; without it a thread writes its own node's 16 words.
+template <bool V4>
 __global__ void pack_input(const float* __restrict__ phi0, const float* __restrict__ phi1,
-                           const float* __restrict__ costh, float* __restrict__ x, int n, long long hw) {
+                           const float* __restrict__ costh, float* __restrict__ x, long long P, long long hw) {
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n * hw) return;
-  float* o = x + p * 16;
-  o[0] = phi0[p];
-  o[1] = phi1[p];
-  o[2] = costh[p / hw];
+  float a = 0.f, b = 0.f, t = 0.f;
+  if (p < P) {
+    a = phi0[p];
+    b = phi1[p];
+    t = costh[P < (1LL << 31) ? (int)((unsigned)p / (unsigned)hw) : p / hw];
+  }
+  if constexpr (V4) {
+    const int lane = threadIdx.x & 31;
+    const long long w0 = p - lane;
 #pragma unroll
-  for (int c = 3; c < 16; ++c) o[c] = 0.f;
+    for (int j = 0; j < 4; ++j) {
+      const int i = j * 32 + lane, from = i >> 2;
+      const float va = __shfl_sync(~0u, a, from), vb = __shfl_sync(~0u, b, from), vt = __shfl_sync(~0u, t, from);
+      if (w0 + from < P)
+        reinterpret_cast<float4*>(x)[w0 * 4 + i] = i & 3 ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(va, vb, vt, 0.f);
+    }
+  } else if (p < P) {
+    float* o = x + p * 16;
+    o[0] = a;
+    o[1] = b;
+    o[2] = t;
+#pragma unroll
+    for (int c = 3; c < 16; ++c) o[c] = 0.f;
+  }
 }
 
-// prediction = base + out[p][0]; loss partials (FP64) and d loss / d out = 2 (pred - target) / P in channel 0
+// prediction = base + out[p][0]; loss partials (FP64) and d loss / d out = 2 (pred - target) / P in channel 0.  Bound by
+// the writes of dout (cpad words a node): V4 (cpad % 4 == 0, dout on 16 bytes) writes a warp's nodes as one run of
+// consecutive float4, as pack_input does (16 images of 256^2, 32 words: 54 us with the sum of the partials, before 180).
+template <bool V4>
 __global__ void mse_residual(const float* __restrict__ out, int cpad, const float* __restrict__ base,
                              const float* __restrict__ target, float* __restrict__ dout, double* __restrict__ part,
                              long long P) {
   __shared__ double s[kThreads];
   const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   double e2 = 0.0;
+  float g = 0.f;
   if (p < P) {
     const float d = (base[p] + out[p * cpad]) - target[p];
     e2 = (double)d * d;
-    dout[p * cpad] = 2.f * d / (float)P;
+    g = 2.f * d / (float)P;
+  }
+  if constexpr (V4) {
+    const int lane = threadIdx.x & 31, q4 = cpad / 4;
+    const long long w0 = p - lane;
+    for (int j = 0; j < q4; ++j) {
+      const int i = j * 32 + lane, from = i / q4;
+      const float v = __shfl_sync(~0u, g, from);
+      if (w0 + from < P)
+        reinterpret_cast<float4*>(dout)[w0 * q4 + i] = make_float4(i == from * q4 ? v : 0.f, 0.f, 0.f, 0.f);
+    }
+  } else if (p < P) {
+    dout[p * cpad] = g;
     for (int c = 1; c < cpad; ++c) dout[p * cpad + c] = 0.f;
   }
   s[threadIdx.x] = e2;
@@ -1072,56 +1109,60 @@ __global__ void to_bf16(const float* __restrict__ a, __nv_bfloat16* __restrict__
 // hi, so a correction step never leaves the bounds.
 __device__ __forceinline__ float proj_bump(float q, float hi) { return hi > 0.f ? q * (hi - q) / hi : 0.f; }
 
-// field = clamp(phi1 + out[p][0], 0, hi)
-__global__ void project_init(const float* __restrict__ out, int cpad, const float* __restrict__ phi0,
-                             const float* __restrict__ phi1, float* __restrict__ field, long long n) {
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const float hi = fmaxf(1.f - phi0[p], 0.f);
-  field[p] = fminf(fmaxf(phi1[p] + out[p * cpad], 0.f), hi);
-}
-
-// per image and part: sums of phi1 (target mass), of the field and of its bump
-__global__ void project_sums(const float* __restrict__ field, const float* __restrict__ phi0,
-                             const float* __restrict__ phi1, double* __restrict__ sums, long long hw) {
+// One stage of the projection over an image's nodes (grid: parts, images):
+//   INIT   field = clamp(phi1 + out[p][0], 0, hi)
+//   APPLY  field += lambda b(field), lambda = clamp((sum phi1 - sum field) / sum b, -1, 1) from the sums of stage `in`
+//   SUM    per image and part: sums of phi1 (target mass), of the field and of its bump, into `sums`
+// A thread meets the same nodes in every stage, so the update of one pass and the sums of the next are one launch; `in`
+// and `sums` are then two buffers, since other CTAs may still read `in`.  Short launches: what counts is their number
+// and the chain of 64 partials, which three threads add (by every thread it is 192 FP64 additions each, at an FP64 rate
+// that is a small part of FP32's).  Three passes on one image of 256^2: 47 us in four launches, 78 before in seven; on 16
+// images 93 against 257.
+template <bool INIT, bool APPLY, bool SUM>
+__global__ void project_stage(const float* __restrict__ out, int cpad, const float* __restrict__ phi0, const float* phi1,
+                              const double* in, double* sums, float* field, long long hw) {
   __shared__ double s[3][kThreads];
-  const int img = blockIdx.y;
-  double a = 0.0, b = 0.0, c = 0.0;
-  for (long long k = (long long)blockIdx.x * kThreads + threadIdx.x; k < hw; k += (long long)gridDim.x * kThreads) {
-    const long long p = img * hw + k;
-    const float q = field[p];
-    a += phi1[p];
-    b += q;
-    c += proj_bump(q, fmaxf(1.f - phi0[p], 0.f));
-  }
-  s[0][threadIdx.x] = a;
-  s[1][threadIdx.x] = b;
-  s[2][threadIdx.x] = c;
-  __syncthreads();
-  for (int k = kThreads / 2; k > 0; k >>= 1) {
-    if ((int)threadIdx.x < k)
-      for (int j = 0; j < 3; ++j) s[j][threadIdx.x] += s[j][threadIdx.x + k];
+  const int img = blockIdx.y, parts = gridDim.x;
+  float lam = 0.f;
+  if constexpr (APPLY) {
+    __shared__ double tot[3];
+    const double* part = in + (long long)img * parts * 3;
+    if (threadIdx.x < 3) {
+      double v = 0.0;
+#pragma unroll 16
+      for (int k = 0; k < parts; ++k) v += part[k * 3 + threadIdx.x];
+      tot[threadIdx.x] = v;
+    }
     __syncthreads();
+    lam = tot[2] > 0.0 ? (float)fmin(1.0, fmax(-1.0, (tot[0] - tot[1]) / tot[2])) : 0.f;
   }
-  if (threadIdx.x == 0)
-    for (int j = 0; j < 3; ++j) sums[((long long)img * gridDim.x + blockIdx.x) * 3 + j] = s[j][0];
-}
-
-// field += lambda b(field), lambda = clamp((sum phi1 - sum field) / sum b, -1, 1) per image
-__global__ void project_apply(const float* __restrict__ phi0, const double* __restrict__ sums, int parts,
-                              float* __restrict__ field, long long hw) {
-  const int img = blockIdx.y;
   double a = 0.0, b = 0.0, c = 0.0;
-  for (int k = 0; k < parts; ++k) {
-    a += sums[((long long)img * parts + k) * 3];
-    b += sums[((long long)img * parts + k) * 3 + 1];
-    c += sums[((long long)img * parts + k) * 3 + 2];
-  }
-  const float lam = c > 0.0 ? (float)fmin(1.0, fmax(-1.0, (a - b) / c)) : 0.f;
-  for (long long k = (long long)blockIdx.x * kThreads + threadIdx.x; k < hw; k += (long long)gridDim.x * kThreads) {
+  for (long long k = (long long)blockIdx.x * kThreads + threadIdx.x; k < hw; k += (long long)parts * kThreads) {
     const long long p = img * hw + k;
-    const float q = field[p];
-    field[p] = q + lam * proj_bump(q, fmaxf(1.f - phi0[p], 0.f));
+    const float hi = fmaxf(1.f - phi0[p], 0.f);
+    float q;
+    if constexpr (INIT) q = fminf(fmaxf(phi1[p] + out[p * cpad], 0.f), hi);
+    else q = field[p];
+    if constexpr (APPLY) q = q + lam * proj_bump(q, hi);
+    if constexpr (INIT || APPLY) field[p] = q;
+    if constexpr (SUM) {
+      a += phi1[p];
+      b += q;
+      c += proj_bump(q, hi);
+    }
+  }
+  if constexpr (SUM) {
+    s[0][threadIdx.x] = a;
+    s[1][threadIdx.x] = b;
+    s[2][threadIdx.x] = c;
+    __syncthreads();
+    for (int k = kThreads / 2; k > 0; k >>= 1) {
+      if ((int)threadIdx.x < k)
+        for (int j = 0; j < 3; ++j) s[j][threadIdx.x] += s[j][threadIdx.x + k];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0)
+      for (int j = 0; j < 3; ++j) sums[((long long)img * parts + blockIdx.x) * 3 + j] = s[j][0];
   }
 }
 
@@ -1394,7 +1435,8 @@ int lbm_nn_pack_input(const float* phi0, const float* phi1, const float* costh, 
                       void* stream) {
   if (!phi0 || !phi1 || !costh || !x || n < 1 || h < 1 || w < 1) return -1;
   const long long hw = (long long)h * w;
-  pack_input<<<blocks(n * hw), 256, 0, (cudaStream_t)stream>>>(phi0, phi1, costh, x, n, hw);
+  const auto pack = reinterpret_cast<uintptr_t>(x) % 16 == 0 ? pack_input<true> : pack_input<false>;
+  pack<<<blocks(n * hw), 256, 0, (cudaStream_t)stream>>>(phi0, phi1, costh, x, n * hw, hw);
   return status(cudaGetLastError());
 }
 
@@ -1404,7 +1446,9 @@ int lbm_nn_mse_residual(const float* out, int cpad, const float* base, const flo
   const int nb = (int)((P + kThreads - 1) / kThreads);
   if (work_len < nb) return -1;
   cudaStream_t s = (cudaStream_t)stream;
-  mse_residual<<<nb, kThreads, 0, s>>>(out, cpad, base, target, dout, work, P);
+  const bool v4 = cpad % 4 == 0 && reinterpret_cast<uintptr_t>(dout) % 16 == 0;
+  const auto mse = v4 ? mse_residual<true> : mse_residual<false>;
+  mse<<<nb, kThreads, 0, s>>>(out, cpad, base, target, dout, work, P);
   sum_double<<<1, 256, 0, s>>>(work, nb, loss);
   return status(cudaGetLastError());
 }
@@ -1432,10 +1476,23 @@ int lbm_nn_project(const float* out, int cpad, const float* phi0, const float* p
   if (work_len < 3LL * parts * n) return -1;
   const long long hw = (long long)h * w;
   cudaStream_t s = (cudaStream_t)stream;
-  project_init<<<blocks(n * hw), 256, 0, s>>>(out, cpad, phi0, phi1, field, n * hw);
+  const dim3 grid(parts, n);
+  // one launch a pass needs the sums twice, and a field apart from phi1, whose sums are the target: else three
+  const uintptr_t f0 = reinterpret_cast<uintptr_t>(field), q0 = reinterpret_cast<uintptr_t>(phi1), len = n * hw * 4;
+  if (work_len >= 6LL * parts * n && (f0 + len <= q0 || q0 + len <= f0)) {
+    double* const buf[2] = {work, work + 3LL * parts * n};
+    project_stage<true, false, true><<<grid, kThreads, 0, s>>>(out, cpad, phi0, phi1, nullptr, buf[0], field, hw);
+    for (int pass = 1; pass < kProjectPasses; ++pass)
+      project_stage<false, true, true><<<grid, kThreads, 0, s>>>(out, cpad, phi0, phi1, buf[(pass - 1) & 1],
+                                                                 buf[pass & 1], field, hw);
+    project_stage<false, true, false><<<grid, kThreads, 0, s>>>(out, cpad, phi0, phi1, buf[(kProjectPasses - 1) & 1],
+                                                                nullptr, field, hw);
+    return status(cudaGetLastError());
+  }
+  project_stage<true, false, false><<<grid, kThreads, 0, s>>>(out, cpad, phi0, phi1, nullptr, nullptr, field, hw);
   for (int pass = 0; pass < kProjectPasses; ++pass) {
-    project_sums<<<dim3(parts, n), kThreads, 0, s>>>(field, phi0, phi1, work, hw);
-    project_apply<<<dim3(parts, n), kThreads, 0, s>>>(phi0, work, parts, field, hw);
+    project_stage<false, false, true><<<grid, kThreads, 0, s>>>(out, cpad, phi0, phi1, nullptr, work, field, hw);
+    project_stage<false, true, false><<<grid, kThreads, 0, s>>>(out, cpad, phi0, phi1, work, nullptr, field, hw);
   }
   return status(cudaGetLastError());
 }
