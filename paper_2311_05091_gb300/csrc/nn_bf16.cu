@@ -21,8 +21,11 @@
 #include <atomic>
 
 #include "../../include/lbm_nn.h"
+#include "nn_plan.cuh"
 
 namespace {
+
+using namespace lbm_nn;
 
 constexpr int kThreads = 128;
 constexpr int kProjectPasses = 3;   // mass-correction passes of lbm_nn_project
@@ -133,56 +136,12 @@ __device__ __forceinline__ void ldg8(const float* p, float* r) {
                : "l"(p));
 }
 
-constexpr int kCvEpi = 8;                          // epilogue warps, two per TMEM lane quarter
-constexpr int kCvMma = kCvEpi;                     // the warp that issues the products
-constexpr int kCvProd = 12;                        // producer warps
-constexpr int kCvThreads = 32 * (kCvEpi + 1 + kCvProd);
-constexpr int kCvBatch = 4;                        // 8-channel groups (32 bytes) a producer thread has in flight
-constexpr int kCvMaxStages = 6;
-constexpr int kCvSmem = 227 * 1024;                // shared memory a CTA may use
-constexpr int kCvHead = 512 + kCvEpi * 4096;       // barriers, epilogue transposition buffers
-
-// How a convolution is cut into work items (host).
-struct FwdPlan {
-  int N, KC;                 // output channels per item, input channels per stage
-  int Wt, pitch, strips;     // columns per item, staged columns, column strips
-  int R, T;                  // rows per item, 128-position tiles per item
-  int Pn;                    // staged positions allocated per channel group (Pn % 8 == 2: conflict-free stores)
-  int stages, stage_bytes, smem, tmem;
-  unsigned mp, mh;           // PosMap's multipliers
-  int blocks, items;         // row blocks of the tall image; items = blocks * strips * (cout / N)
-};
-
 struct FwdArgs {
   const float* x;
   const float* bias;
   float* y;
   int n, h, w, cin, cout, relu;
   FwdPlan p;
-};
-
-// Rows and columns of the flat positions of a block, by multiplication: divisions by the pitch and by the rows h + 1
-// of an image of the tall image (exact: the dividends stay below 2^16, or the quotient below 2).
-struct PosMap {
-  unsigned mp, mh;           // ceil(2^32 / pitch), ceil(2^32 / (h + 1)) or 0: a block spans fewer than h + 1 rows
-  int pitch, h, w;
-  int img0, yy0, x0;         // image and row of the block's first row, image column of position column 0
-  __device__ __forceinline__ void block(long long row0, int col0) {
-    img0 = (int)(row0 / (h + 1));
-    yy0 = (int)(row0 - (long long)img0 * (h + 1));
-    x0 = col0;
-  }
-  // pixel of column c of the block's row r, -1 outside the images
-  __device__ __forceinline__ int pixel(int r, int c) const {
-    const int v = yy0 + r;
-    const int k = mh ? (int)__umulhi((unsigned)v, mh) : (v > h ? 1 : 0);
-    const int yy = v - k * (h + 1), xx = x0 + c;
-    return (yy < h && (unsigned)xx < (unsigned)w) ? ((img0 + k) * h + yy) * w + xx : -1;
-  }
-  __device__ __forceinline__ void split(int q, int& r, int& c) const {
-    r = (int)__umulhi((unsigned)q, mp);
-    c = q - r * pitch;
-  }
 };
 
 template <int N, int KC>
@@ -424,57 +383,6 @@ bool weight_map(CUtensorMap* map, const void* wt, int cin, int cout, int N, int 
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Cuts the convolution into items: among the channel tiles N, the numbers of column strips (of at most 128 columns)
-// and the tiles per item, the least modelled time: waves of one CTA per SM x the largest of the product time (32
-// cycles per M = 128 product up to N = 64, then N / 2), the staging time and the store time (32 bytes per SM and
-// cycle each), plus a fixed latency per item and stage.  Small images get many small items, so that one image of a
-// deep level still reaches half of the SMs; large ones get items of up to 1024 positions, whose halo costs least.
-FwdPlan fwd_plan(int n, int h, int w, int cin, int cout, int sms) {
-  FwdPlan best{};
-  double best_cost = -1.0;
-  const int KC = cin % 32 == 0 ? 32 : 16;
-  const int rows_all = n * (h + 1) - 1;
-  for (int N = 32; N <= 128; N *= 2) {
-    if (cout % N) continue;
-    const int k0 = (w + 127) / 128;
-    for (int k = k0; k <= k0 + 3 && k <= w; ++k) {
-      const int Wt = (w + k - 1) / k, pitch = Wt + 2, strips = (w + Wt - 1) / Wt;
-      for (int T = 1; T * N <= 256; ++T) {
-        if (128 * T < Wt) continue;
-        FwdPlan p{};
-        p.N = N;
-        p.KC = KC;
-        p.Wt = Wt;
-        p.pitch = pitch;
-        p.strips = strips;
-        p.T = T;
-        p.R = std::min((128 * T - Wt) / pitch + 1, rows_all);
-        p.blocks = (rows_all + p.R - 1) / p.R;
-        p.R = (rows_all + p.blocks - 1) / p.blocks;
-        p.mp = (unsigned)(((1ull << 32) + pitch - 1) / pitch);
-        p.mh = p.R + 2 <= h ? 0u : (unsigned)(((1ull << 32) + h) / (h + 1));
-        p.Pn = 128 * T + 2 * pitch + 2;
-        p.Pn += (10 - p.Pn % 8) % 8;                              // Pn % 8 == 2
-        p.stage_bytes = (KC / 8) * p.Pn * 16 + 18 * N * KC;
-        p.stage_bytes = (p.stage_bytes + 511) / 512 * 512;        // the weights' swizzle pattern repeats every 512 bytes
-        p.stages = std::min(kCvMaxStages, (kCvSmem - kCvHead) / p.stage_bytes);
-        if (p.stages < 2) continue;
-        p.smem = kCvHead + p.stages * p.stage_bytes;
-        p.tmem = 32;
-        while (p.tmem < 2 * T * N) p.tmem *= 2;
-        p.items = p.blocks * strips * (cout / N);
-        const double mma = (double)T * 9 * (cin / 16) * std::max(32, N / 2);
-        const double load = ((double)(p.R + 2) * pitch * cin * 4 + 18.0 * cin * N) / 32.0;
-        const double out = (double)T * N * 128 * 4 / 32.0;
-        const double item = std::max(std::max(mma, load), out) + 300.0;
-        const double cost = (double)((p.items + sms - 1) / sms) * item + 400.0 * (cin / KC);
-        if (best_cost < 0 || cost < best_cost) best = p, best_cost = cost;
-      }
-    }
-  }
-  return best;
-}
-
 // ---------------------------------------------------------------------------
 // weight gradient: dw[ky, kx][co][ci] = sum_p dy[p][co] x[p + shift(ky, kx)][ci]
 //
@@ -508,14 +416,6 @@ FwdPlan fwd_plan(int n, int h, int w, int cin, int cout, int sms) {
 // instruction descriptor of kind::f16 with both operands MN-major (transpose bits 15 and 16)
 __host__ __device__ constexpr uint32_t umma_idesc_mn(int m, int n) { return umma_idesc(m, n) | (1u << 15) | (1u << 16); }
 
-constexpr int kWgMaxSlots = 6;
-constexpr int kWgHead = 512;
-constexpr int kWgEpi = 4;                     // warps 0-3: products (one thread of warp 0), then the segment's epilogue
-constexpr int kWgGroups = 3;                  // producer groups of four warps: group g stages steps g, g + 3, ...
-constexpr int kWgGroup = 128, kWgProd = kWgGroups * kWgGroup;
-constexpr int kWgThreads = 32 * kWgEpi + kWgProd;   // 16 warps: 128 registers a thread
-constexpr int kWgBatch = 2;                   // 16-channel groups of each tensor a producer thread has in flight
-
 // barrier `id` of `count` threads with the conjunction of their predicates
 template <int id, int count>
 __device__ __forceinline__ bool meet(bool ok) {
@@ -527,21 +427,6 @@ __device__ __forceinline__ bool meet(bool ok) {
       : "memory");
   return all != 0;
 }
-
-struct WgradPlan {
-  int u_dy;                    // 1: U = dy, V = x; 0: U = x, V = dy
-  int mt, vt, mb;              // channels of U and V per tile; products per b (3 without folding, 2, 1)
-  int utiles, vtiles;
-  int Wt, pitch, strips;
-  int KP, slots;               // positions per step, steps in flight
-  int ulen, rv, vlen;          // plane lengths: U slot; V ring, V plane (ring + 16, padded)
-  int u_bytes, v_bytes, smem, tmem;
-  int seg_steps;               // longest segment
-  unsigned mp, mh;
-  long long len, steps;        // positions and steps of a strip
-  long long chunks;            // partial sums
-  long long bias_chunks, ws_chunks;
-};
 
 struct WgradArgs {
   const float *u, *v;
@@ -1229,98 +1114,6 @@ int lbm_nn_check(void) {
   }
   return 0;
 }
-
-}  // extern "C"
-
-namespace {
-
-constexpr long long kBiasChunk = 4096;
-
-// Tiles and chunks of the weight gradient: the orientation, channel tiles and step length with the least modelled time,
-// (positions per chunk) x the larger of the staging time (12 bytes per SM and cycle, measured for the producer warps)
-// and the product time (shared-memory reads: 32 cycles of U, vt / 4 of V per product).  One CTA per SM, one wave.
-// The workspace keeps at most four sets of partial sums per SM's share of 32 x 32 (up to 64 output channels) or 128 x
-// 32 x one kernel row channel tiles; one set of them is the bias partials' room.
-WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
-  constexpr int sms = 152;
-  const int old_tiles = cout <= 64 ? ((cout + 31) / 32) * ((cin + 31) / 32) : ((cout + 127) / 128) * 3 * ((cin + 31) / 32);
-  const long long most = std::max(1LL, 4LL * sms / old_tiles - 1);
-  // longest float32 chain of one accumulator: the pixels over the partial sums that fit the workspace
-  const long long pixels = (long long)n * h * w;
-  const long long chain = std::max(256LL, pixels * old_tiles / (4 * sms));
-  WgradPlan best{};
-  double best_cost = -1.0;
-  for (int u_dy = 0; u_dy < 2; ++u_dy) {
-    const int cu = u_dy ? cout : cin, cv = u_dy ? cin : cout;
-    for (int mt = 32; mt <= 128; mt *= 2) {
-      if (mt > 32 && cu <= mt / 2) break;
-      const int mb = mt / 32 > 2 ? 3 : mt / 32;
-      for (int vt = 16; vt <= 128; vt += 16) {
-        if (mb * 3 * vt > 512 || (vt > cv && vt > 16)) break;
-        WgradPlan p{};
-        p.u_dy = u_dy;
-        p.mt = mt;
-        p.vt = vt;
-        p.mb = mb;
-        p.utiles = (cu + mt - 1) / mt;
-        p.vtiles = (cv + vt - 1) / vt;
-        const int k = (w + 127) / 128;
-        p.Wt = (w + k - 1) / k;
-        p.pitch = p.Wt + 2;
-        p.strips = (w + p.Wt - 1) / p.Wt;
-        p.len = ((long long)n * (h + 1) - 1) * p.pitch;
-        p.tmem = 32;
-        while (p.tmem < mb * 3 * vt) p.tmem *= 2;
-        for (int kp : {112, 48}) {   // KP + 2 positions of U fill whole passes of a producer group
-          p.KP = kp;
-          // plane lengths for 16-byte stores of a warp's positions and 16-channel groups without bank conflicts
-          // (two groups: 2 mod 4; more: odd)
-          auto pad = [](int len, int groups) {
-            const int want = groups <= 4 ? 2 : 1;   // groups of 8 channels
-            return len + ((want - len) % 8 + 8) % 8;
-          };
-          const int ucopies = mb == 3 ? 1 : 3;
-          p.ulen = pad(mb == 3 ? p.KP + 2 : p.KP, mt / 8);
-          p.u_bytes = (ucopies * mt / 8 * p.ulen * 16 + 127) / 128 * 128;
-          for (p.slots = kWgMaxSlots; p.slots >= 2; --p.slots) {
-            p.rv = p.slots * p.KP + 2 * p.pitch;
-            p.vlen = pad(p.rv + 16, vt / 8);
-            p.v_bytes = vt / 8 * p.vlen * 16;
-            // a product reads 16 planes of U from each block, also where fewer are staged: room for them behind
-            p.smem = kWgHead + p.slots * p.u_bytes + std::max(std::max(p.v_bytes, 16 * p.ulen * 16), 64 * kWgProd);
-            if (p.smem <= kCvSmem) break;
-          }
-          if (p.slots >= 3) break;
-        }
-        if (p.slots < 2) continue;
-        p.steps = (p.len + p.KP - 1) / p.KP;
-        const long long total = p.steps * p.strips, tiles = (long long)p.utiles * p.vtiles;
-        p.chunks = std::max(1LL, std::min(std::min(total, most), sms / tiles));
-        p.chunks = std::min<long long>(p.chunks, 9 * cin);         // room of the bias partials
-        const double waves = (double)((tiles * p.chunks + sms - 1) / sms);
-        const double load = 16.0 * 4 * (std::min(mt, cu) + std::min(vt, cv)) / 12.0;
-        const double mma = mb * 3 * (32.0 + vt / 4.0);
-        const double per = (double)total * p.KP / 16 / p.chunks;
-        const double cost = waves * (per * std::max(load, mma) + 2.0 * p.pitch / 16 * load) + 0.5 * p.chunks * 9;
-        if (best_cost < 0 || cost < best_cost) best = p, best_cost = cost;
-      }
-    }
-  }
-  WgradPlan& p = best;
-  const long long per = (p.steps * p.strips + p.chunks - 1) / p.chunks * p.KP;   // positions per chunk
-  const long long segs = std::max(1LL, (long long)((double)per / (1.1 * chain) + 0.999));
-  p.seg_steps = (int)std::min<long long>(((per + segs - 1) / segs + p.KP - 1) / p.KP, (1 << 22) / p.KP);
-  p.mp = (unsigned)(((1ull << 32) + p.pitch - 1) / p.pitch);
-  const long long rows = (long long)p.seg_steps * p.KP / p.pitch + 5;
-  p.mh = rows <= h ? 0u : (unsigned)(((1ull << 32) + h) / (h + 1));
-  p.bias_chunks = (pixels + kBiasChunk - 1) / kBiasChunk;
-  p.ws_chunks = p.chunks + 1;
-  return best;
-}
-
-}  // namespace
-
-extern "C" {
 
 long long lbm_nn_wgrad_workspace(int n, int h, int w, int cin, int cout) {
   if (n < 1 || h < 1 || w < 1 || cin < 1 || cout < 1) return 0;
