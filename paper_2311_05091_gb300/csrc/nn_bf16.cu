@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a
   if (warp >= kWgEpi) {
     // ---- producers ----
     const int tp = tid - 32 * kWgEpi, tg = tp % kWgGroup, group = tp / kWgGroup;
-    PosMap pm{p.mp, p.mh, p.pitch, a.h, a.w};
+    WgradSegment seg(p, a.h, a.w);
     auto pow2 = [](int g) { return g <= 1 ? 1 : (g <= 2 ? 2 : (g <= 4 ? 4 : 8)); };
     // thread -> (position, 16-channel group), groups fastest; a thread keeps its group for the whole chunk
     const int gu = pow2(nu / 16), gv = pow2(nv / 16);
@@ -496,16 +496,14 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a
     for (int k = 0; k < 16; ++k) bs[k] = 0.f;
     const float* usrc = a.u + u0 + 16 * ku;
     const float* vsrc = a.v + v0 + 16 * kv;
-    // positions are counted from the segment's first; those in [lo, hi) lie in the strip, `off` past the map's row 0
-    int lo = 0, hi = 0, off = 0;
-    // sixteen channels of position q, zero outside the images; dy only on the strip's own columns
+    // sixteen channels of the segment's position q, zero outside the images; dy only on the strip's own columns
     auto fetch = [&](float (&r)[16], const float* src, int c, bool dy, int q, bool on) {
 #pragma unroll
       for (int k = 0; k < 16; ++k) r[k] = 0.f;
-      if (on && q >= lo && q < hi) {
+      if (on && q >= seg.lo && q < seg.hi) {
         int row, col;
-        pm.split(q + off, row, col);
-        const int pix = pm.pixel(row, col);
+        seg.map.split(q + seg.off, row, col);
+        const int pix = seg.map.pixel(row, col);
         if (pix >= 0 && (!dy || (unsigned)(col - 1) < (unsigned)p.Wt)) {
           const float* at = src + (long long)pix * c;
           if (a.wide) {
@@ -560,15 +558,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a
     int it = 0;                                              // steps over all segments
     for (long long t = t0; t < t1;) {
       const long long te = seg_end(t);
-      const int strip = (int)(t / p.steps);
-      const long long first = t % p.steps * p.KP, row0 = first / p.pitch - 2;
       qb = (int)(te - t) * p.KP;
-      // map of the segment: from the row two above its first position's (tall-image rows shifted by two images)
-      pm.block(row0 + 2LL * (a.h + 1), strip * p.Wt - 1);
-      pm.img0 -= 2;
-      off = (int)(first - row0 * p.pitch);
-      lo = (int)max(-first, -(1LL << 30));
-      hi = (int)min(p.len - first, 1LL << 30);
+      seg.start(p, t % p.steps * p.KP, (int)(t / p.steps));
       // the ring restarts at position -pitch: every step of the previous segment is staged (the groups meet first: a
       // phase may only be waited for once the one before it is known to be complete) and its products are done; then
       // the ring's first 2 pitch positions, by all producers

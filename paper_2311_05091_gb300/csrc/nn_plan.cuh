@@ -43,7 +43,16 @@ struct FwdPlan {
 };
 
 // Rows and columns of the flat positions of a block, by multiplication: divisions by the pitch and by the rows h + 1
-// of an image of the tall image (exact: the dividends stay below 2^16, or the quotient below 2).
+// of an image of the tall image.  With m = ceil(2^32 / d) the high word of v m is v / d as long as v (m d - 2^32) < 2^32.
+// By the pitch (at most 130) that holds up to 2^25 positions, by h + 1 where row_multiplier says so.
+// Multiplier of the division by h + 1 for blocks of fewer than `rows` rows: 0 where a block spans fewer than h + 1 (the
+// quotient is 0 or 1), else ceil(2^32 / (h + 1)) if that is exact up to the largest dividend, h + rows.  False if not.
+inline bool row_multiplier(int h, long long rows, unsigned* mh) {
+  const unsigned long long d = h + 1ull, m = ((1ull << 32) + d - 1) / d;
+  *mh = rows <= h ? 0u : (unsigned)m;
+  return rows <= h || (h + (unsigned long long)rows) * (m * d - (1ull << 32)) < (1ull << 32);
+}
+
 struct PosMap {
   unsigned mp, mh;           // ceil(2^32 / pitch), ceil(2^32 / (h + 1)) or 0: a block spans fewer than h + 1 rows
   int pitch, h, w;
@@ -58,7 +67,7 @@ struct PosMap {
     const int v = yy0 + r;
     const int k = mh ? (int)mulhi((unsigned)v, mh) : (v > h ? 1 : 0);
     const int yy = v - k * (h + 1), xx = x0 + c;
-    return (yy < h && (unsigned)xx < (unsigned)w) ? ((img0 + k) * h + yy) * w + xx : -1;
+    return ((unsigned)yy < (unsigned)h && (unsigned)xx < (unsigned)w) ? ((img0 + k) * h + yy) * w + xx : -1;
   }
   LBM_NN_HD void split(int q, int& r, int& c) const {
     r = (int)mulhi((unsigned)q, mp);
@@ -94,7 +103,7 @@ inline FwdPlan fwd_plan(int n, int h, int w, int cin, int cout, int sms) {
         p.blocks = (rows_all + p.R - 1) / p.R;
         p.R = (rows_all + p.blocks - 1) / p.blocks;
         p.mp = (unsigned)(((1ull << 32) + pitch - 1) / pitch);
-        p.mh = p.R + 2 <= h ? 0u : (unsigned)(((1ull << 32) + h) / (h + 1));
+        if (!row_multiplier(h, p.R + 2, &p.mh)) continue;         // never: R <= 342
         p.Pn = 128 * T + 2 * pitch + 2;
         p.Pn += (10 - p.Pn % 8) % 8;                              // Pn % 8 == 2
         p.stage_bytes = (KC / 8) * p.Pn * 16 + 18 * N * KC;
@@ -138,6 +147,23 @@ struct WgradPlan {
   long long len, steps;        // positions and steps of a strip
   long long chunks;            // partial sums
   long long bias_chunks, ws_chunks;
+};
+
+// A segment of a chunk: steps from position `first` (a multiple of KP) of a column strip on, with their map
+struct WgradSegment {
+  PosMap map;
+  int off = 0;               // a position counted from the segment's first lies `off` past the map's row 0
+  int lo = 0, hi = 0;        // the positions in [lo, hi) lie in the strip
+  LBM_NN_HD WgradSegment(const WgradPlan& p, int h, int w) : map{p.mp, p.mh, p.pitch, h, w} {}
+  LBM_NN_HD void start(const WgradPlan& p, long long first, int strip) {
+    // the map starts at the row two above the first position's (tall-image rows shifted by two images)
+    const long long row0 = first / p.pitch - 2;
+    map.block(row0 + 2LL * (map.h + 1), strip * p.Wt - 1);
+    map.img0 -= 2;
+    off = (int)(first - row0 * p.pitch);
+    lo = (int)(-first > -(1LL << 30) ? -first : -(1LL << 30));
+    hi = (int)(p.len - first < (1LL << 30) ? p.len - first : (1LL << 30));
+  }
 };
 
 constexpr long long kBiasChunk = 4096;
@@ -217,8 +243,12 @@ inline WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
   const long long segs = std::max(1LL, (long long)((double)per / (1.1 * chain) + 0.999));
   p.seg_steps = (int)std::min<long long>(((per + segs - 1) / segs + p.KP - 1) / p.KP, (1 << 22) / p.KP);
   p.mp = (unsigned)(((1ull << 32) + p.pitch - 1) / p.pitch);
-  const long long rows = (long long)p.seg_steps * p.KP / p.pitch + 5;
-  p.mh = rows <= h ? 0u : (unsigned)(((1ull << 32) + h) / (h + 1));
+  // with the halo a segment touches fewer than its own positions' rows + 5.  Images of tens of thousands of rows and few
+  // columns: segments shorter than an image where the division by h + 1 would not be exact over several (h > 1500 then)
+  if (!row_multiplier(h, (long long)p.seg_steps * p.KP / p.pitch + 5, &p.mh)) {
+    p.seg_steps = (int)((h - 5LL) * p.pitch / p.KP);
+    row_multiplier(h, (long long)p.seg_steps * p.KP / p.pitch + 5, &p.mh);
+  }
   p.bias_chunks = (pixels + kBiasChunk - 1) / kBiasChunk;
   p.ws_chunks = p.chunks + 1;
   return best;
