@@ -494,8 +494,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a
     float bs[16];
 #pragma unroll
     for (int k = 0; k < 16; ++k) bs[k] = 0.f;
-    const float* usrc = a.u + u0 + 16 * ku;
-    const float* vsrc = a.v + v0 + 16 * kv;
+    const float *usrc = nullptr, *vsrc = nullptr;            // this thread's channels of the segment map's origin
     // sixteen channels of the segment's position q, zero outside the images; dy only on the strip's own columns
     auto fetch = [&](float (&r)[16], const float* src, int c, bool dy, int q, bool on) {
 #pragma unroll
@@ -503,9 +502,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a
       if (on && q >= seg.lo && q < seg.hi) {
         int row, col;
         seg.map.split(q + seg.off, row, col);
-        const int pix = seg.map.pixel(row, col);
-        if (pix >= 0 && (!dy || (unsigned)(col - 1) < (unsigned)p.Wt)) {
-          const float* at = src + (long long)pix * c;
+        const unsigned pix = seg.map.offset(row, col);
+        if (pix != ~0u && (!dy || (unsigned)(col - 1) < (unsigned)p.Wt)) {
+          const float* at = src + (unsigned long long)pix * (unsigned)c;
           if (a.wide) {
             ldg8(at, r);
             ldg8(at + 8, r + 8);
@@ -560,6 +559,8 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a
       const long long te = seg_end(t);
       qb = (int)(te - t) * p.KP;
       seg.start(p, t % p.steps * p.KP, (int)(t / p.steps));
+      usrc = a.u + u0 + 16 * ku + seg.map.origin() * a.cu;
+      vsrc = a.v + v0 + 16 * kv + seg.map.origin() * a.cv;
       // the ring restarts at position -pitch: every step of the previous segment is staged (the groups meet first: a
       // phase may only be waited for once the one before it is known to be complete) and its products are done; then
       // the ring's first 2 pitch positions, by all producers

@@ -42,9 +42,6 @@ struct FwdPlan {
   int blocks, items;         // row blocks of the tall image; items = blocks * strips * (cout / N)
 };
 
-// Rows and columns of the flat positions of a block, by multiplication: divisions by the pitch and by the rows h + 1
-// of an image of the tall image.  With m = ceil(2^32 / d) the high word of v m is v / d as long as v (m d - 2^32) < 2^32.
-// By the pitch (at most 130) that holds up to 2^25 positions, by h + 1 where row_multiplier says so.
 // Multiplier of the division by h + 1 for blocks of fewer than `rows` rows: 0 where a block spans fewer than h + 1 (the
 // quotient is 0 or 1), else ceil(2^32 / (h + 1)) if that is exact up to the largest dividend, h + rows.  False if not.
 inline bool row_multiplier(int h, long long rows, unsigned* mh) {
@@ -53,21 +50,38 @@ inline bool row_multiplier(int h, long long rows, unsigned* mh) {
   return rows <= h || (h + (unsigned long long)rows) * (m * d - (1ull << 32)) < (1ull << 32);
 }
 
+// Rows and columns of the flat positions of a block, by multiplication: divisions by the pitch and by the rows h + 1
+// of an image of the tall image.  With m = ceil(2^32 / d) the high word of v m is v / d as long as v (m d - 2^32) < 2^32.
+// By the pitch (at most 130) that holds up to 2^25 positions, by h + 1 where row_multiplier says so.
 struct PosMap {
   unsigned mp, mh;           // ceil(2^32 / pitch), ceil(2^32 / (h + 1)) or 0: a block spans fewer than h + 1 rows
   int pitch, h, w;
   int img0, yy0, x0;         // image and row of the block's first row, image column of position column 0
   LBM_NN_HD void block(long long row0, int col0) {
-    img0 = (int)(row0 / (h + 1));
-    yy0 = (int)(row0 - (long long)img0 * (h + 1));
+    img0 = (int)(row0 / (h + 1LL));
+    yy0 = (int)(row0 - img0 * (h + 1LL));
     x0 = col0;
   }
-  // pixel of column c of the block's row r, -1 outside the images
+  // whether column c of the block's row r lies in an image: then its row yy and column xx there, and the zero rows k
+  // between the block's first row and it
+  LBM_NN_HD bool inside(int r, int c, unsigned& k, unsigned& yy, unsigned& xx) const {
+    const unsigned v = (unsigned)yy0 + (unsigned)r;
+    k = mh ? mulhi(v, mh) : (v > (unsigned)h ? 1u : 0u);
+    yy = v - k * ((unsigned)h + 1u);
+    xx = (unsigned)x0 + (unsigned)c;
+    return yy < (unsigned)h && xx < (unsigned)w;
+  }
+  // pixel of a launch of fewer than 2^31, -1 outside the images
   LBM_NN_HD int pixel(int r, int c) const {
-    const int v = yy0 + r;
-    const int k = mh ? (int)mulhi((unsigned)v, mh) : (v > h ? 1 : 0);
-    const int yy = v - k * (h + 1), xx = x0 + c;
-    return ((unsigned)yy < (unsigned)h && (unsigned)xx < (unsigned)w) ? ((img0 + k) * h + yy) * w + xx : -1;
+    unsigned k, yy, xx;
+    return inside(r, c, k, yy, xx) ? ((img0 + (int)k) * h + (int)yy) * w + (int)xx : -1;
+  }
+  // the same of a launch of any number, counted from the block's first row, in a block of fewer than 2^32: origin() +
+  // offset(), ~0 outside the images
+  LBM_NN_HD long long origin() const { return ((long long)img0 * h + yy0) * w; }
+  LBM_NN_HD unsigned offset(int r, int c) const {
+    unsigned k, yy, xx;
+    return inside(r, c, k, yy, xx) ? ((unsigned)r - k) * (unsigned)w + xx : ~0u;
   }
   LBM_NN_HD void split(int q, int& r, int& c) const {
     r = (int)mulhi((unsigned)q, mp);
@@ -158,7 +172,7 @@ struct WgradSegment {
   LBM_NN_HD void start(const WgradPlan& p, long long first, int strip) {
     // the map starts at the row two above the first position's (tall-image rows shifted by two images)
     const long long row0 = first / p.pitch - 2;
-    map.block(row0 + 2LL * (map.h + 1), strip * p.Wt - 1);
+    map.block(row0 + 2 * (map.h + 1LL), strip * p.Wt - 1);
     map.img0 -= 2;
     off = (int)(first - row0 * p.pitch);
     lo = (int)(-first > -(1LL << 30) ? -first : -(1LL << 30));
@@ -196,11 +210,11 @@ inline WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
         p.mb = mb;
         p.utiles = (cu + mt - 1) / mt;
         p.vtiles = (cv + vt - 1) / vt;
-        const int k = (w + 127) / 128;
-        p.Wt = (w + k - 1) / k;
+        const int k = (int)((w + 127LL) / 128);
+        p.Wt = (int)((w - 1LL + k) / k);
         p.pitch = p.Wt + 2;
-        p.strips = (w + p.Wt - 1) / p.Wt;
-        p.len = ((long long)n * (h + 1) - 1) * p.pitch;
+        p.strips = (int)((w - 1LL + p.Wt) / p.Wt);
+        p.len = (n * (h + 1LL) - 1) * p.pitch;
         p.tmem = 32;
         while (p.tmem < mb * 3 * vt) p.tmem *= 2;
         for (int kp : {112, 48}) {   // KP + 2 positions of U fill whole passes of a producer group
@@ -243,7 +257,11 @@ inline WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
   const long long segs = std::max(1LL, (long long)((double)per / (1.1 * chain) + 0.999));
   p.seg_steps = (int)std::min<long long>(((per + segs - 1) / segs + p.KP - 1) / p.KP, (1 << 22) / p.KP);
   p.mp = (unsigned)(((1ull << 32) + p.pitch - 1) / p.pitch);
-  // with the halo a segment touches fewer than its own positions' rows + 5.  Images of tens of thousands of rows and few
+  // with the halo a segment touches fewer than its own positions' rows + 5.  Rows of more than 2^17 pixels: segments
+  // shorter than 2^32 pixels (of the six rows that one step touches at most five are below the first: no tensor that
+  // the device holds has seven rows of 2^29 pixels)
+  p.seg_steps = (int)std::max(1LL, std::min<long long>(p.seg_steps, ((1LL << 32) / w - 6) * p.pitch / p.KP));
+  // images of tens of thousands of rows and few
   // columns: segments shorter than an image where the division by h + 1 would not be exact over several (h > 1500 then)
   if (!row_multiplier(h, (long long)p.seg_steps * p.KP / p.pitch + 5, &p.mh)) {
     p.seg_steps = (int)((h - 5LL) * p.pitch / p.KP);

@@ -37,7 +37,8 @@ int main(int argc, char** argv) {
           if (q < seg.lo || q >= seg.hi) continue;
           int r, c;
           seg.map.split(q + seg.off, r, c);
-          const long long got = seg.map.pixel(r, c);
+          const unsigned rel = seg.map.offset(r, c);
+          const long long got = rel == ~0u ? -1 : seg.map.origin() + rel;
           const long long at = first + q, row = at / p.pitch, img = row / (h + 1LL), yy = row % (h + 1LL),
                           xx = at % p.pitch + strip * p.Wt - 1;
           const long long want = yy < h && xx >= 0 && xx < w ? (img * h + yy) * w + xx : -1;
@@ -76,3 +77,11 @@ def walk(tmp_path_factory):
 def test_every_position_maps_to_its_pixel(walk, n, h, w, cin, cout):
     walked, wrong, *_ = walk(n, h, w, cin, cout)
     assert walked > 0 and wrong == 0
+
+
+# 2^31 pixels and more: 128 GB a tensor of 16 channels, half of the device
+@pytest.mark.parametrize("n,h,w", [(1, 65536, 40000), (3, 1 << 20, 1024), (40000, 256, 256), (1 << 20, 1, 2304),
+                                   (1, (1 << 31) - 1, 1), (1, 1, (1 << 31) - 1), (2, (1 << 30) + 77, 1), (5, 3, 150000001)])
+def test_pixels_beyond_32_bits(walk, n, h, w):
+    walked, wrong, far, *_ = walk(n, h, w, 16, 16)
+    assert walked > 0 and wrong == 0 and far == n * h * w - 1
