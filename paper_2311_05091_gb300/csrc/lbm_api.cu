@@ -980,7 +980,7 @@ int lbm_tune(lbm_ctx* c, int trial, int* strips_out) {
   static const int cand[] = {4, 8, 12, 16, 18, 20, 24, 32, 48, 64};
   constexpr int ncand = (int)(sizeof(cand) / sizeof(cand[0]));
   float tile_ms = 1e30f, sweep_ms = 1e30f;
-  if (tile0) e = measure(tile_ms);
+  if (tile0 && e == cudaSuccess) e = measure(tile_ms);
   c->tile = 0;
   for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
     for (int cl = 0; cl < (int)classes.size() && e == cudaSuccess; ++cl) {
