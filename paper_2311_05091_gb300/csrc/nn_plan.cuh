@@ -153,7 +153,10 @@ struct WgradPlan {
   int mt, vt, mb;              // channels of U and V per tile; products per b (3 without folding, 2, 1)
   int utiles, vtiles;
   int Wt, pitch, strips;
-  int KP, slots;               // positions per step, steps in flight
+  int KP;                      // positions per step
+  // Steps in flight, at least kWgGroups: a group that stages step k waits for the products of step k - slots by parity,
+  // which needs those of step k - 2 slots known to be done; what it knows, from its step before, is k - kWgGroups - slots
+  int slots;
   int ulen, rv, vlen;          // plane lengths: U slot; V ring, V plane (ring + 16, padded)
   int u_bytes, v_bytes, smem, tmem;
   int seg_steps;               // longest segment
@@ -228,7 +231,7 @@ inline WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
           const int ucopies = mb == 3 ? 1 : 3;
           p.ulen = pad(mb == 3 ? p.KP + 2 : p.KP, mt / 8);
           p.u_bytes = (ucopies * mt / 8 * p.ulen * 16 + 127) / 128 * 128;
-          for (p.slots = kWgMaxSlots; p.slots >= 2; --p.slots) {
+          for (p.slots = kWgMaxSlots; p.slots >= kWgGroups; --p.slots) {
             p.rv = p.slots * p.KP + 2 * p.pitch;
             p.vlen = pad(p.rv + 16, vt / 8);
             p.v_bytes = vt / 8 * p.vlen * 16;
@@ -236,9 +239,9 @@ inline WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
             p.smem = kWgHead + p.slots * p.u_bytes + std::max(std::max(p.v_bytes, 16 * p.ulen * 16), 64 * kWgProd);
             if (p.smem <= kCvSmem) break;
           }
-          if (p.slots >= 3) break;
+          if (p.slots >= kWgGroups) break;
         }
-        if (p.slots < 2) continue;
+        if (p.slots < kWgGroups) continue;
         p.steps = (p.len + p.KP - 1) / p.KP;
         const long long total = p.steps * p.strips, tiles = (long long)p.utiles * p.vtiles;
         p.chunks = std::max(1LL, std::min(std::min(total, most), sms / tiles));

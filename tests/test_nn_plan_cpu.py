@@ -2,6 +2,7 @@
 walked position by position against plain 64-bit division: images far taller than a segment of the network's levels,
 segments over several images, one and several column strips."""
 import os
+import random
 import subprocess
 
 import pytest
@@ -85,3 +86,12 @@ def test_every_position_maps_to_its_pixel(walk, n, h, w, cin, cout):
 def test_pixels_beyond_32_bits(walk, n, h, w):
     walked, wrong, far, *_ = walk(n, h, w, 16, 16)
     assert walked > 0 and wrong == 0 and far == n * h * w - 1
+
+
+def test_every_plan_has_a_slot_per_producer_group(walk):
+    r = random.Random(11)
+    for _ in range(300):
+        n, h, w = r.randint(1, 20), r.randint(1, 300), r.choice([1, 2, 7, 31, 64, 127, 128, 129, 200, 256, 300, 1000])
+        cin, cout = 16 * r.randint(1, 40), 16 * r.randint(1, 40)
+        walked, wrong, far, segments, slots, longest = walk(n, h, w, cin, cout, 1)
+        assert 3 <= slots <= 6 and segments >= 1 and longest >= 1 and wrong == 0, (n, h, w, cin, cout)
