@@ -22,6 +22,7 @@
 
 #include "../../include/lbm_nn.h"
 #include "nn_plan.cuh"
+#include "nn_wait.cuh"
 
 namespace {
 
@@ -58,7 +59,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 //   epilogue:   reads a finished accumulator (tcgen05.ld), adds the bias, applies the ReLU, transposes through
 //               shared memory and stores whole 128-byte lines.
 // Stages of KC channels form a ring over items; the accumulators have two sets, so an item's products overlap the
-// previous item's epilogue.  Every barrier wait is bounded; a give-up sets g_nn_fault and ends the CTA.
+// previous item's epilogue.  Every barrier wait is bounded (nn_wait.cuh); a give-up sets g_nn_fault and ends the CTA.
 //
 // What bounds it: the wide levels HBM (403 MB for 64 -> 32 on 16 x 256^2: 60 us at copy speed), the deep ones shared
 // memory (an M = 128, K = 16 product reads 4 KB of A, 32 cycles, whatever N) and the pipeline's latency per stage.
@@ -107,26 +108,6 @@ __device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t leader) {
       "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
       " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
       "r"(leader));
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// bounded wait for the completion of phase `parity` of an mbarrier; false when it gave up.  Each poll may suspend the
-// thread for up to 20 us (it wakes when the phase completes), so that waiting warps leave the issue slots to others.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  uint32_t done = 0;
-  for (int it = 0; it < (1 << 20) && !done; ++it)
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(parity), "r"(20000)
-        : "memory");
-  return done != 0;
 }
 
 // eight floats from a 32-byte boundary, through the read-only path
@@ -248,7 +229,8 @@ __global__ void __launch_bounds__(kCvThreads, 1)
     }
     // leave no copy in flight: the last weight tiles issued (landed already unless a wait gave up)
     if (tp == 0)
-      for (int k = 0; k < S && k < it; ++k) (void)mbar_wait(b_w + 8 * ((it - 1 - k) % S), (uint32_t)(((it - 1 - k) / S) & 1));
+      for (int k = 0; k < S && k < it; ++k)
+        if (!mbar_wait(b_w + 8 * ((it - 1 - k) % S), (uint32_t)(((it - 1 - k) / S) & 1))) break;
   } else if (warp == kCvMma) {
     // ---- products: issued by one lane ----
     constexpr uint32_t idesc = umma_idesc(128, N);
@@ -292,7 +274,7 @@ __global__ void __launch_bounds__(kCvThreads, 1)
     // leave no product in flight: the last commits of the stages
     for (int k = 0; k < S && k < it; ++k) {
       const int last = it - 1 - k;
-      (void)mbar_wait(b_empty + 8 * (last % S), (uint32_t)((last / S) & 1));
+      if (!mbar_wait(b_empty + 8 * (last % S), (uint32_t)((last / S) & 1))) break;
     }
   } else {
     // ---- epilogue ----
@@ -723,7 +705,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) conv3x3_wgrad(const WgradArgs a
     }
     if (warp == 0)
       for (int k = 1; k <= S && k <= it; ++k)                // leave no product in flight
-        (void)mbar_wait(b_empty + 8 * ((it - k) % S), (uint32_t)(((it - k) / S) & 1));
+        if (!mbar_wait(b_empty + 8 * ((it - k) % S), (uint32_t)(((it - k) / S) & 1))) break;
   }
   if (!ok) atomicExch(&g_nn_fault, 1u);
   asm volatile("tcgen05.fence::before_thread_sync;");
