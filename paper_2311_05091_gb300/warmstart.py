@@ -123,7 +123,7 @@ class WarmStartNet:
         ws = max(_nn.wgrad_workspace(n, H >> self._lvl(k), Wd >> self._lvl(k), ci, co)
                  for k, (ci, co) in enumerate(self.shapes))
         self.work = torch.empty(ws, dtype=torch.float32, device=self.dev)
-        self.dwork = torch.empty(max(192 * n, (n * H * Wd + 127) // 128 + 8), dtype=torch.float64, device=self.dev)
+        self.dwork = torch.empty(max(384 * n, (n * H * Wd + 127) // 128 + 8), dtype=torch.float64, device=self.dev)
         self.loss = torch.zeros(1, dtype=torch.float64, device=self.dev)
 
     def _lvl(self, k):
