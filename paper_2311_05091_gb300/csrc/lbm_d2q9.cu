@@ -354,7 +354,8 @@ constexpr size_t step_smem_bytes() { return sizeof(StepSmem<D, GT>); }
 // Node update: gradients, forces, velocity, pressure, both collisions and the push stores, from the neighbourhoods of
 // phi1, phi0, mubar_1 and the correction-force product, the chemical-potential differences of the node, the first
 // moment j of its CH populations, its NS populations and its previous step.  Every kernel form of the step calls it
-// with the same values, so that they agree bitwise.
+// with the same values.  Which products it fuses is left to the compiler in each instantiation; that they come out
+// bitwise equal is tested for every form (tests/test_gpu_tile_form.py, tests/test_gpu_tile_rows.py), not ensured here.
 template <bool OBS, typename GT, bool PER>
 __device__ __forceinline__ void collide_node(const StepArgs& a, const InstanceConsts& k, const int b, const int node,
                                              const int x, const int y, const P9& v1, const P9& v0, const P9& vm,
@@ -469,7 +470,7 @@ __device__ __forceinline__ void collide_node(const StepArgs& a, const InstanceCo
 
   // ---- CH collision ----
   {
-        const float emb = k.eta * mub;
+    const float emb = k.eta * mub;
     const float corr = k.corr_scale * (1.f - fdeg);
     // R first moment: d_t(phi1 u) + cs2 * corr * eta grad mubar
     const float Rx = (ph1 * ux - php * uxp) + cs2 * corr * k.eta * gmx;

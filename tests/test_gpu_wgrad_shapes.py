@@ -51,3 +51,15 @@ def test_tall_images_are_exact(lbm_lib, n, h, w, cin, cout):
     dw, db = _wgrad(x, dy)
     ref, rdb = _reference(x, dy)
     assert torch.equal(dw, ref) and torch.equal(db, rdb)
+
+
+# 16-byte loads: either tensor, or both, half a 32-byte sector off; folded and plain channel tiles, one row, strips
+@pytest.mark.parametrize("sx,sdy", [(4, 0), (0, 4), (4, 4)])
+@pytest.mark.parametrize("n,h,w,cin,cout", [(2, 13, 17, 16, 32), (3, 40, 140, 64, 48), (1, 1, 300, 128, 64),
+                                            (2, 33, 31, 80, 144)])
+def test_tensors_on_sixteen_bytes(lbm_lib, n, h, w, cin, cout, sx, sdy):
+    x, dy = _ints((n, h, w, cin), 3, sx), _ints((n, h, w, cout), 4, sdy)
+    assert (x.data_ptr() | dy.data_ptr()) % 32 == 16 and x.is_contiguous()
+    dw, db = _wgrad(x, dy)
+    ref, rdb = _reference(x, dy)
+    assert torch.equal(dw, ref) and torch.equal(db, rdb)
