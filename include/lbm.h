@@ -226,7 +226,10 @@ int lbm_get_instance_shape(const lbm_ctx* ctx, int instance, int* nx, int* ny, i
  * coordinate-descent passes.  The
  * evolving state is saved before and restored after (bitwise), so the call can
  * come at any point after lbm_set_phase.  strips_out (nbatch ints, may be
- * NULL) receives the chosen strip of each instance. */
+ * NULL) receives the fastest strip of each instance: the one in use, unless the
+ * context keeps its tiles.  Then nothing reports that, and passing the strip to
+ * lbm_set_launch (here or on a context of the same shape) selects the slower
+ * sweep: a context whose default is tiles is best left untouched or tuned. */
 int lbm_tune(lbm_ctx* ctx, int trial, int* strips_out);
 
 /* Free all device memory of the context.  Safe on NULL. */

@@ -29,9 +29,10 @@ extern "C" {
 
 /* y[p][co] = act(bias[co] + sum_{tap, ci} x[p + shift(tap)][ci] wt[tap][co][ci]),
  * act = ReLU when relu != 0.  cin a multiple of 16, cout of 32; bias may be NULL.
- * Runs on the tcgen05 tensor cores (FP32 accumulator in tensor memory); a
- * CTA whose bounded wait for its matrix products gives up writes nothing and
- * raises the flag that lbm_nn_check reports. */
+ * Runs on the tcgen05 tensor cores (FP32 accumulator in tensor memory).  A CTA
+ * whose bounded wait (2.1 s) for its copies or matrix products gives up stores
+ * nothing more -- what it had finished stays in y -- and raises the flag that
+ * lbm_nn_check reports. */
 int lbm_nn_conv3x3(const float* x, const void* wt_bf16, const float* bias, float* y, int n, int h, int w,
                    int cin, int cout, int relu, void* stream);
 
@@ -48,7 +49,9 @@ long long lbm_nn_wgrad_workspace(int n, int h, int w, int cin, int cout);
  * (db may be NULL), both overwritten; x and dy are rounded to BF16 as for the
  * forward pass (db sums dy unrounded).  Deterministic: per-chunk partial sums
  * in `work` (work_len floats) are added in a fixed order.  cin a multiple of
- * 16, cout of 16. */
+ * 16, cout of 16.  For finite x: where x is not finite (or rounds to an infinity
+ * in BF16) at the border of an image, or of one of the column strips a wide image
+ * is cut into, the taps that do not reach that value there are NaN as well. */
 int lbm_nn_conv3x3_wgrad(const float* x, const float* dy, float* dw, float* db, float* work, long long work_len,
                          int n, int h, int w, int cin, int cout, void* stream);
 

@@ -325,10 +325,11 @@ int default_strip(const lbm_ctx* c) {
   return (int)std::max(1LL, strip);
 }
 
-// Tile rows of the small-lattice D2Q9 kernel where it is the faster form, else 0: up to 2.5 M nodes (1024^2 x 2: 94 us
-// against 99 of the sweep at its default strip, x 3: 140 against 145, or 131 tuned), and at every size where the rows
-// are not on 16 bytes and the sweep has to copy them word by word (1023^2 x 2: 97 against 106).  Four rows while those
-// CTAs stay below four per SM, else eight.
+// Tile rows of the small-lattice D2Q9 kernel where it is the faster form, else 0: at every size where the rows are not on
+// 16 bytes and the sweep has to copy them word by word (1023^2 x 2: 97 us against 106), and up to 2.5 M nodes.  There the
+// sweep at its best strip overtakes it, not the sweep at its default strip (1024^2 x 2: 94 against 99 at the default,
+// x 3: 140 against 145, but 131 tuned; x 5: 229 against 212 tuned), so an untuned context of 1024^2 x 3 nodes would still
+// be 3 % faster with tiles.  Four rows while those CTAs stay below four per SM, else eight.
 int default_tile(const lbm_ctx* c) {
   if (c->lattice != LBM_D2Q9 || c->multi) return 0;
   if (c->total > 2500000 && c->nx % 4 == 0) return 0;

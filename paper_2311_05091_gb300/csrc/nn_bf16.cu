@@ -387,8 +387,8 @@ bool weight_map(CUtensorMap* map, const void* wt, int cin, int cout, int N, int 
 // the float32 chains of the sums should get (and at strip ends); the first segment's sums are written to part[z], the
 // others added.  Producer warps load and round, and sum dy for the bias gradient (unrounded, in a fixed order), in
 // three groups that stage every third step each; one lane issues the products; then four warps move the sums out.
-// An activation or gradient that is not finite makes its whole channel's gradient NaN: the products of the halo
-// columns multiply it by zero.
+// Where x is not finite next to a halo column or a zero row, the products with dy = 0 there make NaN of taps that do not
+// reach that value otherwise.
 //
 // What bounds it: the producers' instructions and load latency on the wide levels (HBM: 40 us for 32 -> 32 on
 // 16 x 256^2), the products elsewhere.  Measured (GB300, 16 images, with the sums and the bias gradient): 32 -> 32 on

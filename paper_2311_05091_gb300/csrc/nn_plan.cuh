@@ -188,15 +188,16 @@ constexpr long long kBiasChunk = 4096;
 // Tiles and chunks of the weight gradient: the orientation, channel tiles and step length with the least modelled time,
 // (positions per chunk) x the larger of the staging time (12 bytes per SM and cycle, measured for the producer warps)
 // and the product time (shared-memory reads: 32 cycles of U, vt / 4 of V per product).  One CTA per SM, one wave.
-// The workspace keeps at most four sets of partial sums per SM's share of 32 x 32 (up to 64 output channels) or 128 x
-// 32 x one kernel row channel tiles; one set of them is the bias partials' room.
+// The size of the workspace, which callers keep, bounds the chunks: four sets of partial sums per SM's share of channel
+// tiles, 32 x 32 (up to 64 output channels) or 128 x 32 x one kernel row, the last set being the bias partials' room, and
+// cout floats per 4096 pixels, which nothing uses.  It does not depend on the device: it is asked for without one.
 inline WgradPlan wgrad_plan(int n, int h, int w, int cin, int cout) {
-  constexpr int sms = 152;
-  const int old_tiles = cout <= 64 ? ((cout + 31) / 32) * ((cin + 31) / 32) : ((cout + 127) / 128) * 3 * ((cin + 31) / 32);
-  const long long most = std::max(1LL, 4LL * sms / old_tiles - 1);
+  constexpr int sms = 152;     // of a GB300
+  const int ws_tiles = cout <= 64 ? ((cout + 31) / 32) * ((cin + 31) / 32) : ((cout + 127) / 128) * 3 * ((cin + 31) / 32);
+  const long long most = std::max(1LL, 4LL * sms / ws_tiles - 1);
   // longest float32 chain of one accumulator: the pixels over the partial sums that fit the workspace
   const long long pixels = (long long)n * h * w;
-  const long long chain = std::max(256LL, pixels * old_tiles / (4 * sms));
+  const long long chain = std::max(256LL, pixels * ws_tiles / (4 * sms));
   WgradPlan best{};
   double best_cost = -1.0;
   for (int u_dy = 0; u_dy < 2; ++u_dy) {
