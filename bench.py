@@ -426,8 +426,8 @@ def time_to_equilibrium(L, stream, size, total, every, tol_deg=0.5, flags=0, tun
     area relation).  The equilibrium angle of an instance is its last sample;
     its time to equilibrium is the first sample from which every later sample
     stays within tol_deg of it (at least five samples, else None).  Wall time
-    = steps x the device time per step of the same lattice, at the strip the
-    library's autotuner picks for it (strips change no result bit).
+    = steps x the device time per step of the same lattice, in the form the
+    library's autotuner keeps for it: tiles, or the fastest strip (neither changes a result bit).
     """
     import torch
     wl = make_workload("disk1024x5", size)
